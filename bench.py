@@ -410,11 +410,12 @@ def n0_sweep_study(g, torch, dev_in, outs, shapes, sweep=None):
 
 def residual_roofline(g, torch, n=16384, k=4096, reps=3):
     """The sliced FP64-class residual (the mixed path's dominant kernel) at
-    n = 16384, k = 4096, as each refinement sweep runs it: L's digit planes
-    come from the plan (trsm_plan_mixed), X is sliced inside the timed call,
-    then the stream kernel forms R = B - L X.  bf16 MMA flops (P(P+1)/2
-    plane pairs x 2 x n^2/2 x k) per call / CUDA-event time, against the bf16
-    tensor peak; the slicing of X (about 1 % of the call) counts as time."""
+    n = 16384, k = 4096, as each refinement sweep runs it: L's residues come
+    from the plan (trsm_plan_mixed), those of X are made inside the timed
+    call, then the products form R = B - L X.  bf16 MMA flops (14 or 15
+    moduli x 2 x n^2/2 x k for the classes of seven and eight planes) per
+    call / CUDA-event time, against the bf16 tensor peak; the residues of X
+    count as time."""
     import ctypes
     lib = g.load_library()
     L = torch.tril(torch.rand(n, n, dtype=torch.float64, device="cuda") * 2 - 1) / n
@@ -446,9 +447,9 @@ def residual_roofline(g, torch, n=16384, k=4096, reps=3):
             torch.cuda.synchronize()
             ts.append(a.elapsed_time(b))
         ms = statistics.median(ts)
-        flops = planes * (planes + 1) / 2 * float(n) * n * k
+        flops = {7: 14, 8: 15}[planes] * float(n) * n * k
         achieved = flops / (ms * 1e-3) / 1e12
-        out[f"planes{planes}"] = {"bound": "tensor", "kernel": "sliced stream_kernel (with the slicing of X)",
+        out[f"planes{planes}"] = {"bound": "tensor", "kernel": "rns_product_kernel (with the residues of X)",
                                   "ms": round(ms, 3), "achieved": round(achieved, 1), "peak": burst,
                                   "unit": "TFLOP/s", "frac": round(achieved / burst, 4), "peak_source": src,
                                   "err_flag": int(err.item())}
@@ -567,21 +568,22 @@ def schedules_study(g, torch, dev_in, outs, shapes, n0s, reps=3, stream=None, fp
     return out
 
 
-def sliced_mma_flops(n, k, nb):
-    """BF16 tensor-core flops of one sliced solve: 36 digit-plane pairs for
-    every product; the updates W(T_{i+1}) -= L(T_{i+1}, S_i) X_i take
+def sliced_mma_flops(n, k, nb, products=36):
+    """BF16 tensor-core flops of one sliced solve that takes `products` BF16
+    products for every FP64-class one (15 moduli; 36 pairs of eight 6-bit
+    digits); the updates W(T_{i+1}) -= L(T_{i+1}, S_i) X_i take
     2 (n - (i+1) nb) nb k each, the diagonal multiplies 2 m_i^2 k / 2 (the
     strictly lower part of each inverted block)."""
     N = -(-n // nb)
     upd = sum(2.0 * (n - (i + 1) * nb) * nb * k for i in range(N - 1))
     diag = sum(float(min(nb, n - i * nb)) ** 2 * k for i in range(N))
-    return 36.0 * (upd + diag)
+    return float(products) * (upd + diag)
 
 
 def sliced_study(g, torch, data, dev_in, outs, shapes, reps=3):
-    """The sliced schedule (both matrix multiplies as FP64-class digit-sliced
+    """The sliced schedule (both matrix multiplies as FP64-class integer
     products on the BF16 tensor cores) on the FP64 sweep shapes at its own
-    block size: plan (inversion, then digit planes) and solve times, TFLOP/s
+    block size: plan (inversion, then residues) and solve times, TFLOP/s
     (n^2 k), the relative error of sampled columns against the oracle, and
     the tensor-core roofline of the solve."""
     import oracle
@@ -613,7 +615,7 @@ def sliced_study(g, torch, data, dev_in, outs, shapes, reps=3):
         want = oracle.forward_subst_columns(L, B, cols)
         got = X[:, torch.from_numpy(cols).cuda()].cpu().numpy()
         err = float(np.max(np.abs(got - want)) / np.max(np.abs(want)))
-        mma = sliced_mma_flops(n, k, nb) / (ms * 1e-3) / 1e12
+        mma = sliced_mma_flops(n, k, nb, 15) / (ms * 1e-3) / 1e12
         rows[f"{n}x{k}"] = [nb, round(plan_ms, 2), round(planes_ms, 2), round(ms, 2),
                             round(float(n) * n * k / (ms * 1e-3) / 1e12, 2), _sig(err), round(mma / burst, 3)]
         p.destroy()
@@ -631,7 +633,7 @@ def serving_study(g, torch, nL=256, rates=(100, 300, 600, 1200, 2400), per_rate=
     mixed-precision plan (split-fp16 updates), and half of the requests on
     them ask for the refined mixed-precision solve (tol 1e-12; diagonal
     multiplies as `mixed_s`: two tf32 planes on the tensor cores) instead of
-    FP64.  The same L also carry the sliced schedule's digit planes, and an
+    FP64.  The same L also carry the sliced schedule's residues, and an
     FP64 request of at least sliced_min_flops n^2 k flops is solved by the
     sliced schedule (FP64-class, on the tensor cores) instead of joining a
     batch.  Reports solves/s and p50/p99 latency, overall and for the mixed
@@ -692,14 +694,14 @@ def serving_study(g, torch, nL=256, rates=(100, 300, 600, 1200, 2400), per_rate=
 
 def run_case(args):
     """Single kernels for profiling (no JSON bench line):
-    sliced:N:K[:P]   the tensor-core residual R = B - L X with P (7 or 8)
-                     digit planes, twice;
+    sliced:N:K[:P]   the tensor-core residual R = B - L X in the class
+                     of P (7 or 8) planes, twice;
     mixed:N:K:N0[:I[:S]]  one mixed-precision refined solve (graded diagonal,
                      c = 2); inner I = 0 tf32, 1 bf16, 2 split bf16, 3 split
                      fp16; S = 1 for the FP32 diagonal-block multiply, 2, 3
                      or 4 for the tensor-core one with 3, 2 or 1 tf32 planes;
     sched:N:K:N0     the sliced schedule of the FP64 solve (well-conditioned
-                     L), its digit planes made first, then two solves;
+                     L), its residues made first, then two solves;
     engine:M:N:K     the bf16 tensor-core GEMM self-test, twice;
     batch:COUNT:BITS[:N0] one batched launch of COUNT systems of the
                      batching workload in FP64 (BITS = 64) or FP32 (32),

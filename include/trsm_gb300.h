@@ -55,15 +55,18 @@ extern "C" {
  * powers of two into fp16's range and the update undoes both */
 #define TRSM_INNER_FP16X3 4
 /* Residual of the mixed-precision solve. */
-#define TRSM_RESIDUAL_SLICED 0   /* FP64-class, bf16 tensor cores, 7 integer digit planes */
+/* The sliced residuals run on the bf16 tensor cores in integer arithmetic: L
+ * to 48 bits of each (row, 2048-wide chunk) maximum, X to 42 bits of each
+ * (column, chunk) maximum in the seven-plane class, 48 in the eight-plane
+ * class (35 in the classes of five and six), exact products. */
+#define TRSM_RESIDUAL_SLICED 0   /* FP64-class: the seven-plane class */
 #define TRSM_RESIDUAL_FP64 1     /* FP64 fused multiply-add                                */
-#define TRSM_RESIDUAL_SLICED8 2  /* as SLICED with 8 digit planes: ~2^-49 instead of ~2^-43 */
+#define TRSM_RESIDUAL_SLICED8 2  /* the eight-plane class: ~2^-50 instead of ~2^-45 */
 #define TRSM_RESIDUAL_ADAPTIVE 3 /* SLICED until the updates stagnate above tol or their contraction
                                     stalls (an update ten times above the last contraction's
                                     prediction), then SLICED8 */
-/* As ADAPTIVE, but an early residual takes 5 or 6 digit planes (15 or 21
- * plane products instead of 28; about 2^-31 and 2^-37 of |B| + |L||X|)
- * while the iterate's error, estimated from the last update and its
+/* As ADAPTIVE, but an early residual takes the class of 5 or 6 planes (13
+ * tensor-core products instead of 14; about 2^-38 of |B| + |L||X|) while the iterate's error, estimated from the last update and its
  * contraction, is far above what they resolve; 7 planes after that, 8 once
  * the updates stagnate. */
 #define TRSM_RESIDUAL_PROGRESSIVE 4
@@ -132,14 +135,15 @@ int trsm_solve(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, dou
  *   TRSM_SCHED_SLICED         It-Inv-TRSM in its right-looking order with
  *                             both matrix multiplies, X_i = L~_ii W_i and
  *                             W(T_{i+1}) -= L(T_{i+1}, S_i) X_i, on the BF16
- *                             tensor cores: each factor is split into eight
- *                             6-bit integer digit planes with a power-of-two
- *                             exponent per row (per row and block column for
- *                             L), the 36 plane pairs of weight >= 2^-42 are
- *                             multiplied with exact FP32 sums, and the
- *                             results are combined and applied in FP64.
- *                             Each product carries about 2^-49 of |A| |B|
- *                             (an FP64-class result, not FP64 rounding).
+ *                             tensor cores: each factor is rounded to 48
+ *                             bits below a power-of-two exponent per row (per
+ *                             row and block column for L), its residues
+ *                             modulo 15 small primes and prime powers are
+ *                             multiplied with exact FP32 sums, and the exact
+ *                             integer products are put together from their
+ *                             residues and applied in FP64.  Each product
+ *                             carries about 2^-49 of |A| |B| (an FP64-class
+ *                             result, not FP64 rounding).
  *                             Needs trsm_plan_sliced on the plan first
  *                             (else TRSM_EINVAL) and k <= 5242800; X_dev
  *                             may equal B_dev with ldx == ldb.
@@ -154,11 +158,11 @@ int trsm_solve_schedule(trsm_handle_t h, const double* B_dev, int64_t k, int64_t
 
 /* trsm_plan_sliced — adds the data of TRSM_SCHED_SLICED to a plan (no
  * counterpart in the paper, which assumes exact arithmetic: this is the
- * digit splitting of Ozaki, Ogita, Oishi & Rump, 2012, applied to the two
- * matrix multiplies of It-Inv-TRSM, Section 6.2).  From the plan's L~ it
- * makes eight bf16 digit planes of L off the diagonal blocks (16 n^2 bytes)
- * and of the rows of the inverted diagonal blocks (16 n n0 bytes), counted
- * by trsm_plan_device_bytes and freed by trsm_destroy.  The block order must
+ * integer modular form of Ozaki's splitting, Ozaki, Uchino & Imamura, 2025,
+ * applied to the two matrix multiplies of It-Inv-TRSM, Section 6.2).  From
+ * the plan's L~ it makes the bf16 residues modulo 15 moduli of L off the
+ * diagonal blocks (15 n (n + n0) bytes) and of the rows of the inverted
+ * diagonal blocks (30 n n0 bytes), counted by trsm_plan_device_bytes and freed by trsm_destroy.  The block order must
  * be a multiple of 64 and at most 2048, or the plan a single block (n0 >= n)
  * of order at most 2048 (else TRSM_EINVAL).  A second call is a no-op.
  * Synchronous.  Errors: TRSM_EINVAL, TRSM_ENOMEM, TRSM_ECUDA. */
@@ -206,7 +210,7 @@ int trsm_solve_noalloc(trsm_handle_t h, const double* B_dev, int64_t k, int64_t 
  *   - FP32 copies of the plan's inverted diagonal blocks L~_ii (n x n0
  *     floats), for the FP32 diagonal-block multiply, and three tf32 planes
  *     of them (3 n x n0 floats), for the tensor-core one;
- *   - eight 6-bit integer digit planes of the strictly lower L, for the
+ *   - the residues modulo 15 moduli of the strictly lower L, for the
  *     FP64-class residual.
  *   L_dev : the same matrix the plan was made from (n x n, ldl >= n).
  * Synchronous.  Errors: TRSM_EINVAL, TRSM_ENOMEM, TRSM_ECUDA. */
@@ -226,7 +230,7 @@ int trsm_plan_mixed(trsm_handle_t h, const double* L_dev, int64_t ldl, int inner
  *              block), optionally or-ed with TRSM_SOLVE_S_FP32 or
  *              one of TRSM_SOLVE_S_TC, _TC2, _TC1.  The
  *              residual's accuracy sets the attainable error: about
- *              cond * 2^-43 (SLICED), cond * 2^-49 (SLICED8), cond * 2^-53
+ *              cond * 2^-45 (SLICED), cond * 2^-50 (SLICED8), cond * 2^-53
  *              (FP64), with cond the componentwise condition of the system
  *              (the sliced residuals are componentwise only within a
  *              2048-row chunk of X: a solution whose entries span many
@@ -350,13 +354,13 @@ int trsm_plan_sizes(trsm_handle_t h, int64_t* n, int64_t* n0, int64_t* nblocks);
 const double* trsm_plan_lt(trsm_handle_t h, int64_t* ldt);
 
 /* Device bytes the plan holds: L~ and, after trsm_plan_mixed, the
- * mixed-precision data (panels, digit planes, diagonal blocks).  0 for a
+ * mixed-precision data (panels, residues, diagonal blocks).  0 for a
  * null handle.  No counterpart in the paper: memory accounting for callers
  * that admit work against an HBM budget. */
 size_t trsm_plan_device_bytes(trsm_handle_t h);
 
 /* Workspace memory.  The per-call scratch of every solve, plan and batch
- * run (working copy of B, digit planes, counters) comes from a
+ * run (working copy of B, residues, counters) comes from a
  * stream-ordered memory pool the library owns, one per device.  Memory a
  * call frees stays reserved in the pool for the next call (the device's
  * default pool would unmap it at each synchronisation and the next call

@@ -118,7 +118,7 @@ def choose_n0(n, dtype="f64", table=None):
 
 def tune_schedule(plan, B, X=None, reps=2):
     """Times the schedules of the blocked solve on this system (the sliced
-    one only where the plan's block order allows it; its digit planes are
+    one only where the plan's block order allows it; its residues are
     made before the timing); returns (fastest name, {name: ms})."""
     times = {}
     for sched in binding.SCHEDULES:

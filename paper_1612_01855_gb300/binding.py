@@ -178,7 +178,7 @@ class Plan:
         _check(lib.trsm_plan_sizes(self._h, ctypes.byref(n), ctypes.byref(n0), ctypes.byref(nb)),
                "trsm_plan_sizes")
         self.n, self.n0, self.nblocks = n.value, n0.value, nb.value
-        self.sliced = False  # digit planes of the sliced schedule (trsm_plan_sliced)
+        self.sliced = False  # residues of the sliced schedule (trsm_plan_sliced)
 
     @property
     def handle(self):
@@ -311,7 +311,7 @@ SCHEDULES = {"dag": 0, "right-looking": 1, "recursive": 2, "sliced": 3}
 
 
 def trsm_plan_sliced(plan):
-    """Adds the digit planes of the sliced schedule to a plan (synchronous;
+    """Adds the residues of the sliced schedule to a plan (synchronous;
     a no-op when they are there)."""
     if getattr(plan, "sliced", False):
         return
@@ -325,7 +325,7 @@ def trsm_solve_schedule(plan, B, X=None, schedule="dag"):
     """trsm_solve with a chosen schedule: "dag" (default persistent
     kernel), "right-looking" (the paper's B~ loop with look-ahead),
     "recursive" (Rec-TRSM) or "sliced" (both matrix multiplies as
-    FP64-class digit-sliced tensor-core products; its plan data is made on
+    FP64-class integer tensor-core products; its plan data is made on
     first use).  Asynchronous."""
     torch = _torch()
     if schedule == "sliced":

@@ -19,7 +19,7 @@ struct trsm_plan_s {
   int* status = nullptr;  // sticky device status of solves
   int device = 0;
   trsm::MixedPlan* mixed = nullptr;    // low-precision data (trsm_plan_mixed), or null
-  trsm::SlicedPlan* sliced = nullptr;  // digit planes of the sliced schedule (trsm_plan_sliced), or null
+  trsm::SlicedPlan* sliced = nullptr;  // residues of the sliced schedule (trsm_plan_sliced), or null
 };
 
 namespace trsm {
@@ -28,7 +28,7 @@ namespace trsm {
 // Device bytes of the plan's mixed-precision data (0 without it).
 size_t mixed_bytes(const trsm_plan_s* h);
 void mixed_release(trsm_plan_s* h);
-// The same for the digit planes of the sliced schedule.
+// The same for the residues of the sliced schedule.
 size_t sliced_bytes(const trsm_plan_s* h);
 void sliced_release(trsm_plan_s* h);
 // X = L^-1 B by the sliced schedule (sched_sliced.cu): B is copied first, so

@@ -24,9 +24,9 @@
 // multiply (from its maximum), the GEMM undoing both through a device
 // factor on alpha.
 //
-// The residual is either the digit-sliced tensor-core product of sliced.cu
-// (relative to |B| + |L||X|: about 2^-43 with seven planes, about 2^-49
-// with eight; or seven until the updates stagnate above tol or their
+// The residual is either the residue-number-system tensor-core product of
+// rns.cu (relative to |B| + |L||X|: about 2^-45 in the seven-plane class,
+// about 2^-50 in the eight-plane class; or seven until the updates stagnate above tol or their
 // contraction stalls, then eight) or
 // a plain FP64 DFMA product.
 #include <cuda_bf16.h>
@@ -40,7 +40,7 @@
 
 #include "fp64_tile.cuh"
 #include "internal.h"
-#include "sliced.h"
+#include "rns.h"
 #include "tc_host.h"
 #include "trsm_gb300.h"
 
@@ -52,8 +52,8 @@ struct MixedPlan {
   void* panels = nullptr;   // low-precision L(T_{i+1}, S_i), i = 0..N-2, row-major [rows][n0p]
   double* diag = nullptr;   // diag(L)
   double* dblk = nullptr;   // the original diagonal blocks of L, N x n0 x n0 (FP64 residual)
-  void* lsl = nullptr;      // digit planes of the strictly lower L
-  SlicedOperand Ls;
+  void* lsl = nullptr;      // residue planes of the strictly lower L
+  RnsOperand Ls;
   int* panel_exp = nullptr; // split fp16: panel i is stored times 2^panel_exp[i]
   float* dinv32 = nullptr;  // FP32 copies of the inverted diagonal blocks L~_ii, N x n0 x n0 (ld n0)
   float* dinv_tc = nullptr; // tf32 hi / mid / lo planes of the inverted blocks, K-major: block b at
@@ -854,7 +854,7 @@ extern "C" int trsm_plan_mixed(trsm_handle_t h, const double* L_dev, int64_t ldl
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&mp->diag), sizeof(double) * n);
   if (e == cudaSuccess)
     e = cudaMalloc(reinterpret_cast<void**>(&mp->dblk), sizeof(double) * static_cast<size_t>(N * n0 * n0));
-  const size_t lbytes = trsm::sliced_operand_bytes(n, n);
+  const size_t lbytes = trsm::rns_operand_bytes(n, n, trsm::kChunk, true);
   if (e == cudaSuccess) e = cudaMalloc(&mp->lsl, lbytes);
   mp->bytes = esz * panel_elems + sizeof(double) * n + sizeof(double) * static_cast<size_t>(N * n0 * n0) + lbytes;
   double* tmp = nullptr;
@@ -911,8 +911,8 @@ extern "C" int trsm_plan_mixed(trsm_handle_t h, const double* L_dev, int64_t ldl
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    mp->Ls = trsm::sliced_operand_view(mp->lsl, n, n);
-    e = trsm::slice_lower_rows(L_dev, ldl, n, mp->Ls, tmp, s);
+    mp->Ls = trsm::rns_operand_view(mp->lsl, n, n, trsm::kChunk, true);
+    e = trsm::rns_lower_rows(L_dev, ldl, n, mp->Ls, tmp, s);
   }
   if (tmp) trsm::ws_free(tmp, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -951,7 +951,7 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   const int64_t ld = trsm::align4(n);
   const size_t esz = trsm::mode_bytes(mode);
 
-  // workspace: R, D (FP64), W (FP32), Dt (low precision), X digit planes, norms, error word
+  // workspace: R, D (FP64), W (FP32), Dt (low precision), residues of X and of the products, norms, error word
   size_t off = 0;
   const size_t oR = off;
   off = trsm::align256(off + sizeof(double) * ld * k);
@@ -962,9 +962,9 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   const size_t oDt = off;
   off = trsm::align256(off + esz * n0p * k);
   const size_t oXs = off;
-  off = trsm::align256(off + trsm::sliced_operand_bytes(k, n));
+  off = trsm::align256(off + trsm::rns_operand_bytes(k, n));
   const size_t oPart = off;
-  off = trsm::align256(off + trsm::sliced_partial_bytes(n, k));
+  off = trsm::align256(off + (residual != TRSM_RESIDUAL_FP64 ? trsm::rns_scratch_bytes(n, k) : 0));
   const size_t oNorm = off;
   off = trsm::align256(off + 2 * sizeof(unsigned long long) + sizeof(int));
   const size_t oDmax = off;  // per block row: max |D_i| (split fp16 scaling)
@@ -980,7 +980,8 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   double* D = reinterpret_cast<double*>(ws + oD);
   float* W = reinterpret_cast<float*>(ws + oW);
   void* Dt = ws + oDt;
-  trsm::SlicedOperand Xs = trsm::sliced_operand_view(ws + oXs, k, n);
+  trsm::RnsOperand Xs = trsm::rns_operand_view(ws + oXs, k, n);
+  const trsm::RnsScratch scratch = trsm::rns_scratch_view(ws + oPart, n, k);
   unsigned long long* norms = reinterpret_cast<unsigned long long*>(ws + oNorm);
   int* err = reinterpret_cast<int*>(ws + oNorm + 2 * sizeof(unsigned long long));
   unsigned long long* dmax = reinterpret_cast<unsigned long long*>(ws + oDmax);
@@ -993,7 +994,7 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   // The first sweep solves with B itself (its W is made from B_dev) and
   // sets X = D without reading X.
   double best = HUGE_VAL, prev = HUGE_VAL, prev2 = HUGE_VAL;  // the last two updates
-  // digit planes of the sliced residual: the adaptive mode starts with seven
+  // accuracy class of the sliced residual: the adaptive mode starts with seven
   // and moves to eight when the updates stagnate above tol or their
   // contraction stalls; the progressive
   // mode chooses five, six or seven from the iterate's estimated error (then
@@ -1169,10 +1170,10 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
     }
     // ---- R = B - L X ----
     if (residual != TRSM_RESIDUAL_FP64) {
-      e = trsm::slice_rows(X_dev, ldx, Xs, s);
+      if (it == 1) e = trsm::rns_scratch_clear(scratch, s);
+      if (e == cudaSuccess) e = trsm::rns_rows(X_dev, ldx, n, Xs, trsm::rns_class(planes), s);
       if (e == cudaSuccess)
-        e = trsm::sliced_residual(mp->Ls, mp->diag, 0, Xs, X_dev, ldx, B_dev, ldb, R, ld, ws + oPart, true,
-                                  planes, err, s);
+        e = trsm::rns_residual(mp->Ls, mp->diag, Xs, X_dev, ldx, B_dev, ldb, R, ld, planes, scratch, err, s);
     } else {
       dim3 g(static_cast<unsigned>((n + trsm::TILE - 1) / trsm::TILE),
              static_cast<unsigned>((k + trsm::TILE - 1) / trsm::TILE));
@@ -1202,16 +1203,17 @@ extern "C" int trsm_residual_plan(trsm_handle_t h, const double* X_dev, int64_t 
     return TRSM_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t n = h->n;
-  const size_t xb = trsm::align256(trsm::sliced_operand_bytes(k, n));
-  const size_t pb = trsm::align256(trsm::sliced_partial_bytes(n, k));
+  const size_t xb = trsm::align256(trsm::rns_operand_bytes(k, n));
+  const size_t pb = trsm::align256(trsm::rns_scratch_bytes(n, k));
   unsigned char* buf = nullptr;
   cudaError_t e = trsm::ws_alloc(reinterpret_cast<void**>(&buf), xb + pb, s);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TRSM_ENOMEM : TRSM_ECUDA;
-  const trsm::SlicedOperand Xs = trsm::sliced_operand_view(buf, k, n);
-  e = trsm::slice_rows(X_dev, ldx, Xs, s);
+  const trsm::RnsOperand Xs = trsm::rns_operand_view(buf, k, n);
+  const trsm::RnsScratch sc = trsm::rns_scratch_view(buf + xb, n, k);
+  e = trsm::rns_scratch_clear(sc, s);
+  if (e == cudaSuccess) e = trsm::rns_rows(X_dev, ldx, n, Xs, trsm::rns_class(planes), s);
   if (e == cudaSuccess)
-    e = trsm::sliced_residual(h->mixed->Ls, h->mixed->diag, 0, Xs, X_dev, ldx, B_dev, ldb, R_dev, ldr, buf + xb, true,
-                              planes, err_dev, s);
+    e = trsm::rns_residual(h->mixed->Ls, h->mixed->diag, Xs, X_dev, ldx, B_dev, ldb, R_dev, ldr, planes, sc, err_dev, s);
   trsm::ws_free(buf, s);
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -21,7 +21,7 @@ pays for the blocked solve (Algorithm It-Inv-TRSM, Section 6.2).  The loop:
   multiplies: "tc2" (default: two tf32 planes on the tensor cores), "tc",
   "fp32" or "fp64" (the DFMA pipe, which then dominates the solve);
 * with `sliced_min_flops` set, an FP64 request of at least that many n^2 k
-  flops whose plan carries the sliced schedule's digit planes
+  flops whose plan carries the sliced schedule's residues
   (`trsm_plan_sliced`) waits in a third queue and is solved alone on a slot
   by the sliced schedule (FP64-class products on the tensor cores, 10-20x
   the DFMA rate on large systems): the largest requests, which set the
@@ -192,15 +192,25 @@ class Server:
     @staticmethod
     def request_bytes(n, k, mixed=False, sliced_block=0):
         if sliced_block:
-            # X, and the sliced solve's workspace: W (FP64), the digit planes
-            # of one block row of W and of X (eight bf16 planes each)
-            return 16 * n * k + 2 * 16 * k * sliced_block + 4 * k + (1 << 16)
+            # X, and the sliced solve's workspace: W (FP64), the residues of
+            # one block row (15 bf16 values each) and those of the products
+            return 16 * n * k + 30 * k * (sliced_block + 64) + Server._product_bytes(n, k) + 4 * k + (1 << 16)
         if mixed:
             # X, and the refinement's workspace: R, D (FP64), W (FP32), the
-            # eight digit planes of X (bf16), the float-float partial sums
-            return (8 + 8 + 8 + 4 + 16 + 8) * n * k + (1 << 16)
+            # residues of X (15 bf16 values) and those of the products
+            return (8 + 8 + 8 + 4 + 30) * n * k + Server._product_bytes(n, k) + (1 << 16)
         # B and X, the working copy W inside the batch workspace, counters
         return 3 * 8 * n * k + 4 * ((n + 31) // 32) * ((k + 31) // 32) * 2 + 4096
+
+    @staticmethod
+    def _product_bytes(n, k):
+        """Residues of the products in flight: 15 bytes per output of the
+        padded 128 x 64, 128 or 256 tiles, at most 512 MiB or one column of
+        tiles, and the tiles' counters."""
+        width = 64 if k <= 64 else 128 if k <= 128 else 256
+        rows = -(-n // 128) * 128
+        cap = max(rows * width, (512 << 20) // 15)
+        return 15 * min(rows * -(-k // width) * width, cap)
 
     def submit(self, req):
         plan = self.plans[req.lid]
