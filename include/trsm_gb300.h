@@ -113,7 +113,10 @@ int trsm_plan(const double* L_dev, int64_t n, int64_t ldl, int64_t n0, void* str
  *           undefined.
  *   k     : number of right-hand sides, k >= 0 (k == 0 is a no-op).
  * Asynchronous on `stream`; it allocates its workspace (n x k doubles plus
- * dependency counters) stream-ordered and frees it stream-ordered.  A
+ * dependency counters; none for small solves that run by columns)
+ * stream-ordered and frees it stream-ordered.  The form of the solve (tile
+ * tasks over all columns, or columns dealt to the SMs) follows from n, k and
+ * the block order; the result is the same bits either way.  A
  * device-side wait that times out is reported by trsm_sync_status.
  * Errors (immediate): TRSM_EINVAL, TRSM_ENOMEM, TRSM_ECUDA. */
 int trsm_solve(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, double* X_dev,

@@ -74,6 +74,22 @@ cudaError_t solve_enqueue(const double* Lt, int64_t ldt, int64_t n, int64_t n0, 
                           int64_t k, int64_t ldb, double* X, int64_t ldx, void* ws,
                           int* status_dev, cudaStream_t s);
 
+// The solve by columns (solve_cols.cu): CW columns per group, S CTAs per
+// group; use: whether it is expected to be faster than the tile tasks.
+struct ColPlan {
+  bool use = false;
+  int S = 0, CW = 0, stages = 0;
+  size_t smem = 0;
+};
+ColPlan col_plan(int64_t n, int64_t n0, int64_t k);
+cudaError_t col_solve(const ColPlan& p, const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B, int64_t k,
+                      int64_t ldb, double* X, int64_t ldx, int* status_dev, cudaStream_t s);
+
+// The solve by whichever of the two is expected to be faster; ws may be null
+// when col_plan says use.
+cudaError_t solve_any(const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B, int64_t k, int64_t ldb,
+                      double* X, int64_t ldx, void* ws, int* status_dev, cudaStream_t s);
+
 // Device status word and device ordinal of a plan (for entry points that
 // live outside api.cu).
 int* plan_status_word(trsm_handle_t h);
