@@ -6,15 +6,25 @@
 // bottom-up over all blocks at once: the two half inversions of a node are
 // independent (the paper runs them on disjoint processor sub-grids), so on
 // one GPU every node of the same height across every diagonal block is
-// processed by one launch.  Leaves (order <= 32) are inverted by one warp
+// processed by one launch.  Leaves (order <= 32) are inverted by one CTA
 // each; each internal node costs two batched tile-GEMM launches per height:
 //   T      = -(L22^-1 * L21)   (the first multiply of RecTriInv)
 //   L21^-1 =  T * L11^-1       (the second multiply)
 // exploiting the triangular factor to skip K ranges that multiply zeros.
+//
+// Bound by the FP64 pipe (2 multiply-adds per SM and clock), so what counts
+// is that every SM has work to the end.  The tiles of a launch differ in
+// their K range (32 to h), and are launched longest first, at most four CTAs
+// to an SM (enough to keep its pipe full, as in the blocked solve): the SMs
+// that finish early find short tiles left.  With every tile resident from
+// the start, in row order, the pipe was busy half of the time: n = 8192, n0 =
+// 512, us: the last height's products 458 + 328, all of them 1155, the leaves
+// (a warp each, 850 dependent FP64 instructions of 64 clocks) 55.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
 
+#include "fp64_leaf.cuh"
 #include "fp64_tile.cuh"
 #include "internal.h"
 
@@ -34,85 +44,103 @@ struct LeafDesc {
 struct NodeDesc {
   int64_t off;    // element offset of the node's top-left corner
   int64_t toff;   // element offset of this node's T (r x h, ld r) in scratch
-  int64_t tile0;  // first flat tile of this node within its launch
   int32_t h;      // order of L11 (a multiple of LEAF)
   int32_t r;      // order of L22
   int32_t tr;     // ceil(r / TILE)
   int32_t tc;     // h / TILE
 };
 
-// One warp per leaf: lane j computes column j of the inverse by column
-// substitution on L y = e_j, then the block is written back coalesced.
-__global__ void __launch_bounds__(128) leaf_inverse_kernel(double* __restrict__ A, int64_t ld,
-                                                           const LeafDesc* __restrict__ leaves,
-                                                           int nleaves,
-                                                           unsigned long long* __restrict__ sing) {
-  __shared__ double ls[4][LEAF][LEAF + 1];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int leaf = blockIdx.x * 4 + warp;
-  if (leaf >= nleaves) return;  // whole warps only; no block-wide barrier below
-  const LeafDesc d = leaves[leaf];
-  double* base = A + d.off;
-  const int m = d.m;
-  for (int c = 0; c < LEAF; ++c) {
-    double v = 0.0;
-    if (lane < m && c < m && lane >= c) v = base[(int64_t)c * ld + lane];
-    ls[warp][lane][c] = v;
-  }
-  __syncwarp();
-  if (lane < m) {
-    const double dl = ls[warp][lane][lane];
-    if (dl == 0.0 || !isfinite(dl)) atomicMin(sing, (unsigned long long)(d.row0 + lane));
-  }
-  double y[LEAF];
+struct FirstSingular {
+  unsigned long long* sing;
+  __device__ void operator()(int64_t row) const { atomicMin(sing, static_cast<unsigned long long>(row)); }
+};
+
+// One CTA per leaf, in place.
+__global__ void __launch_bounds__(NTHREADS) leaf_inverse_kernel(double* __restrict__ A, int64_t ld,
+                                                                const LeafDesc* __restrict__ leaves,
+                                                                unsigned long long* __restrict__ sing) {
+  __shared__ double ls[LEAF][LEAF + 1], tb[16][17];
+  const LeafDesc d = leaves[blockIdx.x];
+  leaf_invert_block<double>(A + d.off, ld, d.m, A + d.off, ld, ls, tb, FirstSingular{sing}, d.row0);
+}
+
+// acc = A(rows [0, m), K [kbeg, kend)) B(K [kbeg, kend), 32 columns), as
+// tile_mma of fp64_tile.cuh with the next chunk's loads issued before the
+// current chunk's multiply-adds (two shared-memory buffers, one barrier per
+// chunk).  kTri: A's last chunk is its diagonal one, A(r, kend - m + ...) = 0
+// to the right of row r: warp w, which holds rows 8 w to 8 w + 7, stops it
+// after 8 (w + 1) steps.
+struct PipeSmem {
+  TileSmem buf[2];
+};
+template <bool kTri>
+__device__ __forceinline__ void tile_product(const double* __restrict__ A, int64_t lda, const double* __restrict__ B,
+                                             int64_t ldb, int m, int64_t kbeg, int64_t kend, PipeSmem& sm,
+                                             double (&acc)[TM][TN]) {
+  constexpr int kPer = KCH * TILE / NTHREADS;  // elements of either operand per thread and chunk
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int ty = tid >> 4, tx = tid & 15;
+  double ra[kPer], rb[kPer];
+  auto load = [&](int64_t k0) {
 #pragma unroll
-  for (int r = 0; r < LEAF; ++r) y[r] = (r == lane) ? 1.0 : 0.0;
-#pragma unroll
-  for (int l = 0; l < LEAF; ++l) {
-    if (l < m) {
-      y[l] = y[l] / ls[warp][l][l];
-#pragma unroll
-      for (int r = l + 1; r < LEAF; ++r) y[r] = fma(-ls[warp][r][l], y[l], y[r]);
+    for (int it = 0; it < kPer; ++it) {
+      const int64_t ta = k0 + w + 4 * it, tb = k0 + lane;
+      ra[it] = (lane < m && ta < kend) ? A[ta * lda + lane] : 0.0;
+      rb[it] = tb < kend ? B[static_cast<int64_t>(w + 4 * it) * ldb + tb] : 0.0;
     }
-  }
-  __syncwarp();
+  };
+  auto store = [&](TileSmem& b) {
 #pragma unroll
-  for (int r = 0; r < LEAF; ++r) ls[warp][r][lane] = y[r];  // column `lane` of the inverse
-  __syncwarp();
-  if (lane < m) {
-    for (int c = 0; c < m; ++c) base[(int64_t)c * ld + lane] = ls[warp][lane][c];
+    for (int it = 0; it < kPer; ++it) {
+      b.a[w + 4 * it][lane] = ra[it];
+      b.b[lane][w + 4 * it] = rb[it];
+    }
+  };
+  zero_acc(acc);
+  load(kbeg);
+  store(sm.buf[0]);
+  __syncthreads();
+  int cur = 0;
+  for (int64_t k0 = kbeg; k0 < kend; k0 += KCH) {
+    const bool more = k0 + KCH < kend;
+    if (more) load(k0 + KCH);
+    const TileSmem& b = sm.buf[cur];
+    const int steps = static_cast<int>(imin64(KCH, kend - k0));
+    const int end = kTri && !more ? min(steps, 8 * w + 8) : steps;
+#pragma unroll 8
+    for (int kk = 0; kk < end; ++kk) {
+      double av[TM], bv[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) av[i] = b.a[kk][ty * TM + i];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) bv[j] = b.b[kk][tx * TN + j];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+    }
+    if (more) store(sm.buf[cur ^ 1]);  // last read before the previous barrier
+    __syncthreads();
+    cur ^= 1;
   }
 }
 
-__device__ __forceinline__ int find_node(const NodeDesc* nodes, int nnodes, int64_t t) {
-  int lo = 0, hi = nnodes - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (nodes[mid].tile0 <= t) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// T = -(L22^-1 * L21): one TILE x TILE tile of T per CTA.
-__global__ void __launch_bounds__(NTHREADS) combine_first_kernel(const double* __restrict__ A,
-                                                                 int64_t ld,
-                                                                 const NodeDesc* __restrict__ nodes,
-                                                                 int nnodes,
+// T = -(L22^-1 * L21): one TILE x TILE tile of T per CTA.  Row tile a of the
+// lower triangular L22^-1 only meets K < (a + 1) TILE: blockIdx.y counts the
+// row tiles from the last.  blockIdx.x: node and column tile, `cols` of them
+// per node.
+__global__ void __launch_bounds__(NTHREADS) combine_first_kernel(const double* __restrict__ A, int64_t ld,
+                                                                 const NodeDesc* __restrict__ nodes, int cols,
                                                                  double* __restrict__ T) {
-  __shared__ TileSmem sm;
-  const int64_t t = blockIdx.x;
-  const NodeDesc nd = nodes[find_node(nodes, nnodes, t)];
-  const int64_t q = t - nd.tile0;
-  const int a = (int)(q % nd.tr), b = (int)(q / nd.tr);
+  __shared__ PipeSmem sm;
+  const NodeDesc nd = nodes[blockIdx.x / cols];
+  const int a = nd.tr - 1 - static_cast<int>(blockIdx.y), b = blockIdx.x % cols;
+  if (a < 0 || b >= nd.tc) return;
   const double* L22inv = A + nd.off + (int64_t)nd.h * ld + nd.h;
   const double* L21 = A + nd.off + nd.h;
-  const int m = min(TILE, nd.r - a * TILE);
   double acc[TM][TN];
-  zero_acc(acc);
-  // L22^-1 is lower triangular: row tile a only meets K < (a+1)*TILE.
-  tile_mma_fp64<false, false>(L22inv + a * TILE, ld, L21 + (int64_t)b * TILE * ld, ld, m, TILE, 0,
-                              min((a + 1) * TILE, nd.r), sm, acc);
+  tile_product<true>(L22inv + a * TILE, ld, L21 + (int64_t)b * TILE * ld, ld, min(TILE, nd.r - a * TILE), 0,
+                     min((a + 1) * TILE, nd.r), sm, acc);
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   double* To = T + nd.toff;
 #pragma unroll
@@ -127,24 +155,19 @@ __global__ void __launch_bounds__(NTHREADS) combine_first_kernel(const double* _
   }
 }
 
-// L21^-1 = T * L11^-1, written over L21.
+// L21^-1 = T * L11^-1, written over L21.  Column tile b of the lower
+// triangular L11^-1 only meets K >= b TILE: blockIdx.y is the column tile.
+// blockIdx.x: node and row tile, `rows` of them per node.
 __global__ void __launch_bounds__(NTHREADS) combine_second_kernel(double* __restrict__ A, int64_t ld,
-                                                                  const NodeDesc* __restrict__ nodes,
-                                                                  int nnodes,
+                                                                  const NodeDesc* __restrict__ nodes, int rows,
                                                                   const double* __restrict__ T) {
-  __shared__ TileSmem sm;
-  const int64_t t = blockIdx.x;
-  const NodeDesc nd = nodes[find_node(nodes, nnodes, t)];
-  const int64_t q = t - nd.tile0;
-  const int a = (int)(q % nd.tr), b = (int)(q / nd.tr);
-  const double* Tn = T + nd.toff;
-  const double* L11inv = A + nd.off;
-  const int m = min(TILE, nd.r - a * TILE);
+  __shared__ PipeSmem sm;
+  const NodeDesc nd = nodes[blockIdx.x / rows];
+  const int a = blockIdx.x % rows, b = blockIdx.y;
+  if (a >= nd.tr || b >= nd.tc) return;
   double acc[TM][TN];
-  zero_acc(acc);
-  // L11^-1 is lower triangular: column tile b only meets K >= b*TILE.
-  tile_mma_fp64<false, false>(Tn + a * TILE, nd.r, L11inv + (int64_t)b * TILE * ld, ld, m, TILE,
-                              (int64_t)b * TILE, nd.h, sm, acc);
+  tile_product<false>(T + nd.toff + a * TILE, nd.r, A + nd.off + (int64_t)b * TILE * ld, ld,
+                      min(TILE, nd.r - a * TILE), (int64_t)b * TILE, nd.h, sm, acc);
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   double* Out = A + nd.off + nd.h;
 #pragma unroll
@@ -272,16 +295,14 @@ cudaError_t invert_diag_blocks(double* A, int64_t ld, const std::vector<DiagBloc
     if (b.m > 0) tb.build(b.off, b.m, b.row0);
   if (tb.leaves.empty()) return cudaSuccess;
 
-  // Flat tile numbering per height and T scratch offsets (scratch reused
-  // across heights: heights run one after another on the stream).
+  // T scratch offsets (scratch reused across heights: heights run one after
+  // another on the stream).
   int64_t scratch_elems = 0;
   size_t node_total = 0;
   for (auto& lvl : tb.by_height) {
-    int64_t tile = 0, toff = 0;
+    int64_t toff = 0;
     for (NodeDesc& nd : lvl) {
-      nd.tile0 = tile;
       nd.toff = toff;
-      tile += (int64_t)nd.tr * nd.tc;
       toff += (int64_t)nd.r * nd.h;
     }
     scratch_elems = std::max(scratch_elems, toff);
@@ -315,17 +336,27 @@ cudaError_t invert_diag_blocks(double* A, int64_t ld, const std::vector<DiagBloc
   }
   if (e == cudaSuccess) {
     const LeafDesc* d_leaves = (const LeafDesc*)desc;
-    const int nleaves = (int)tb.leaves.size();
-    leaf_inverse_kernel<<<(nleaves + 3) / 4, 128, 0, s>>>(A, ld, d_leaves, nleaves, sing_dev);
+    leaf_inverse_kernel<<<(unsigned)tb.leaves.size(), NTHREADS, 0, s>>>(A, ld, d_leaves, sing_dev);
     count_launch();
     e = cudaGetLastError();
     const NodeDesc* d_nodes = (const NodeDesc*)((unsigned char*)desc + leaf_bytes);
+    // shared memory that four CTAs of the products take up
+    constexpr int kPad = 56 * 1024 - (int)sizeof(PipeSmem);
+    if (e == cudaSuccess && node_total > 0) {
+      e = cudaFuncSetAttribute(combine_first_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(combine_second_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPad);
+    }
     for (auto& lvl : tb.by_height) {
       if (e != cudaSuccess) break;
-      const int nn = (int)lvl.size();
-      const int64_t tiles = lvl.back().tile0 + (int64_t)lvl.back().tr * lvl.back().tc;
-      combine_first_kernel<<<(unsigned)tiles, NTHREADS, 0, s>>>(A, ld, d_nodes, nn, T);
-      combine_second_kernel<<<(unsigned)tiles, NTHREADS, 0, s>>>(A, ld, d_nodes, nn, T);
+      const unsigned nn = (unsigned)lvl.size();
+      int tr = 1, tc = 1;
+      for (const NodeDesc& nd : lvl) {
+        tr = std::max(tr, nd.tr);
+        tc = std::max(tc, nd.tc);
+      }
+      combine_first_kernel<<<dim3(nn * tc, tr), NTHREADS, kPad, s>>>(A, ld, d_nodes, tc, T);
+      combine_second_kernel<<<dim3(nn * tr, tc), NTHREADS, kPad, s>>>(A, ld, d_nodes, tr, T);
       count_launch(2);
       e = cudaGetLastError();
       d_nodes += nn;
