@@ -160,21 +160,24 @@ struct StoreF64MaxEpi {
     const int c0 = tn * BN + sl * 16;
     const int ncol = (r < M) ? min(16, N - c0) : 0;
     double* base = D + static_cast<int64_t>(c0) * ldd + r;
-    unsigned long long mb = 0;
+    // the maximum as the bits of |v| in FP32, one conversion at the end
+    // (conversions to double go through the narrow FP64 pipe)
+    uint32_t mf = 0;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       if (j >= ncol) continue;
       base[static_cast<int64_t>(j) * ldd] = static_cast<double>(v[j]);
-      const float a = fabsf(v[j]);
-      const unsigned long long b = (a != a) ? 0x7FF8000000000000ull
-                                            : static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(a)));
-      mb = b > mb ? b : mb;
+      const uint32_t b = __float_as_uint(v[j]) & 0x7FFFFFFFu;
+      mf = b > mf ? b : mf;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long b = __shfl_xor_sync(0xffffffffu, mb, o);
-      mb = b > mb ? b : mb;
+      const uint32_t b = __shfl_xor_sync(0xffffffffu, mf, o);
+      mf = b > mf ? b : mf;
     }
+    const unsigned long long mb = mf > 0x7F800000u ? 0x7FF8000000000000ull  // a NaN
+                                                   : static_cast<unsigned long long>(__double_as_longlong(
+                                                         static_cast<double>(__uint_as_float(mf))));
     if ((threadIdx.x & 31) == 0 && mb) atomicMax(dmax, mb);
   }
   __device__ void slab_done(State&, int, int, int, int, int) const {}
@@ -257,13 +260,16 @@ namespace {
 // P tf32 planes of each factor: P = 3 takes the six products above, P = 2
 // the three of weight 2^-11 and above (hi hi, hi mid, mid hi: about 2^-21
 // of the product), P = 1 the hi planes alone (tf32, about 2^-11).  A stage
-// holds P planes of both operands (32 KB each): two stages at P = 3, three
-// at P = 2 and P = 1 (two CTAs per SM at P = 1).
-template <int P>
+// holds P planes of both operands (32 KB each at BN = 128): two stages at P =
+// 3, three at P = 2 and P = 1 (two CTAs per SM at P = 1).  Few tiles take 32
+// columns (20 KB a plane, up to four stages): a 128-column tile's FP64 stores and
+// its operand loads are most of a short product's time (M = K = 256, N =
+// 128, P = 2: 19 us with 2 CTAs, 10 us with 8).
+template <int P, int BN>
 cudaError_t split_tf32_tri(const float* A, int64_t lda, int64_t a_plane, const float* B, int64_t ldb,
                            int64_t b_plane, double* D, int64_t ldd, int64_t M, int64_t N, int64_t K,
                            unsigned long long* dmax, int* err, cudaStream_t s) {
-  constexpr int BN = 128, STAGES = P == 3 ? 2 : 3;
+  constexpr int STAGES = BN < 128 ? (P == 3 ? 3 : 4) : P == 3 ? 2 : 3;
   using Cfg = TileCfg<true, BN, P, P, 1, STAGES>;
   using Pairs = std::conditional_t<P == 3, Split3Pairs, std::conditional_t<P == 2, SplitPairs, OnePair>>;
   using Epi = StoreF64MaxEpi<BN, Cfg::KB>;
@@ -279,10 +285,16 @@ cudaError_t gemm_split_tf32_tri(const float* A, int64_t lda, int64_t a_plane, co
                                 int64_t b_plane, double* D, int64_t ldd, int64_t M, int64_t N, int64_t K,
                                 int planes, unsigned long long* dmax, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
+  const bool few = (M + 127) / 128 * ((N + 31) / 32) <= device_sm_count();
+  auto run = [&](auto p) {
+    constexpr int P = decltype(p)::value;
+    return few ? split_tf32_tri<P, 32>(A, lda, a_plane, B, ldb, b_plane, D, ldd, M, N, K, dmax, err, s)
+               : split_tf32_tri<P, 128>(A, lda, a_plane, B, ldb, b_plane, D, ldd, M, N, K, dmax, err, s);
+  };
   switch (planes) {
-    case 1: return split_tf32_tri<1>(A, lda, a_plane, B, ldb, b_plane, D, ldd, M, N, K, dmax, err, s);
-    case 2: return split_tf32_tri<2>(A, lda, a_plane, B, ldb, b_plane, D, ldd, M, N, K, dmax, err, s);
-    case 3: return split_tf32_tri<3>(A, lda, a_plane, B, ldb, b_plane, D, ldd, M, N, K, dmax, err, s);
+    case 1: return run(std::integral_constant<int, 1>());
+    case 2: return run(std::integral_constant<int, 2>());
+    case 3: return run(std::integral_constant<int, 3>());
     default: return cudaErrorInvalidValue;
   }
 }
