@@ -108,6 +108,43 @@ cudaError_t ws_alloc(T** p, size_t bytes, cudaStream_t s) {
   return ws_alloc(reinterpret_cast<void**>(p), bytes, s);
 }
 
+// A kernel launched with programmatic dependence on the one before it in the
+// stream: it may be set up while that one still runs, and must call
+// grid_dependency_wait before it touches global memory (in every CTA, before
+// any return, so that its end implies the end of its predecessors).  The
+// kernel before it lets it start early by calling grid_launch_dependents: the
+// short element-wise kernels of a chain do, so that the tensor-core kernel
+// after them finds its barriers and tensor memory set up.  The tensor-core
+// kernels do not: CTAs that wait beside them slow them down (n = 16384, k =
+// 256, sliced, us: 1298 without any of this, 1327 with both kinds letting go
+// early, 1218 with the element-wise ones alone; refined n = 3000, k = 128:
+// 1295, 965, 925), and a CTA that waits must not hold tensor memory that one
+// of them still has to get.
+// cluster: CTAs per cluster (1: none).
+template <class... KArgs, class... Args>
+cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             unsigned cluster, Args&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 // Unique id of the calling thread's current CUDA context (0 if none is
 // current or the driver entry points are unavailable): caches of device
 // addresses and pools are keyed by it, so that they are remade after a

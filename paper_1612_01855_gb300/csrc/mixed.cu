@@ -219,6 +219,8 @@ __device__ __forceinline__ double scale_pow2(double x, int n) {
 __global__ void pack_dt_f16_kernel(const double* __restrict__ D, int64_t ldd, int64_t s0, int m, int64_t k,
                                    int64_t n0p, const unsigned long long* __restrict__ dmax, const int* panel_exp,
                                    __half* __restrict__ Dt, float* __restrict__ gscale) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int sd = 14 - exp_above(*dmax);
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *gscale = ldexpf(1.f, -(*panel_exp + sd));
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
@@ -297,6 +299,8 @@ __global__ void pack_inv_tf32_kernel(const double* __restrict__ Lt, int64_t ldt,
 template <int P>
 __global__ void pack_w_tf32_kernel(const float* __restrict__ W, int64_t ldw, int64_t s0, int m, int64_t k,
                                    int64_t n0p, float* __restrict__ Wt) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (t >= n0p) return;
   const int64_t plane = k * n0p;
@@ -316,6 +320,8 @@ __global__ void pack_w_tf32_kernel(const float* __restrict__ W, int64_t ldw, int
 template <int P>
 __global__ void pack_w_tf32_vec_kernel(const float* __restrict__ W, int64_t ldw, int64_t s0, int m, int64_t k,
                                        int64_t n0p, float* __restrict__ Wt) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int64_t t = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x);
   if (t >= n0p) return;
   const int64_t plane = k * n0p;
@@ -351,6 +357,8 @@ __global__ void pack_w_tf32_vec_kernel(const float* __restrict__ W, int64_t ldw,
 template <int kMode>
 __global__ void pack_dt_kernel(const double* __restrict__ D, int64_t ldd, int64_t s0, int m, int64_t k, int64_t n0p,
                                typename LowP<kMode>::T* __restrict__ Dt) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= m) return;
   for (int64_t col = blockIdx.y; col < k; col += gridDim.y)
@@ -387,6 +395,8 @@ __global__ void extract_diag_kernel(const double* __restrict__ L, int64_t ldl, i
 template <bool kVec>
 __global__ void to_float_kernel(const double* __restrict__ R, int64_t ldr, float* __restrict__ W,
                                 int64_t ldw, int64_t n, int64_t k) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int64_t i = 2 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x);
   if (i >= n) return;
   const bool pair = i + 1 < n;
@@ -700,6 +710,8 @@ template <bool kVec, bool kFirst>
 __global__ void correct_kernel(double* __restrict__ X, int64_t ldx, const double* __restrict__ D,
                                int64_t ldd, int64_t n, int64_t k,
                                unsigned long long* __restrict__ norms) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   constexpr unsigned long long kAbs = ~(1ull << 63);
   unsigned long long dm = 0, xm = 0;
   auto one = [&](int64_t j, int64_t i) {
@@ -965,10 +977,10 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   off = trsm::align256(off + trsm::rns_operand_bytes(k, n));
   const size_t oPart = off;
   off = trsm::align256(off + (residual != TRSM_RESIDUAL_FP64 ? trsm::rns_scratch_bytes(n, k) : 0));
-  const size_t oNorm = off;
-  off = trsm::align256(off + 2 * sizeof(unsigned long long) + sizeof(int));
-  const size_t oDmax = off;  // per block row: max |D_i| (split fp16 scaling)
-  off = trsm::align256(off + sizeof(unsigned long long) * N);
+  const size_t oErr = off;
+  off = trsm::align256(off + sizeof(int));
+  const size_t oDmax = off;  // per block row: max |D_i| (split fp16 scaling); then max |D|, max |X|
+  off = trsm::align256(off + sizeof(unsigned long long) * (N + 2));
   const size_t oGscale = off;
   off = trsm::align256(off + sizeof(float) * N);
   const size_t oWt = off;  // tf32 planes of W_i (tensor-core diagonal multiply)
@@ -982,9 +994,9 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   void* Dt = ws + oDt;
   trsm::RnsOperand Xs = trsm::rns_operand_view(ws + oXs, k, n);
   const trsm::RnsScratch scratch = trsm::rns_scratch_view(ws + oPart, n, k);
-  unsigned long long* norms = reinterpret_cast<unsigned long long*>(ws + oNorm);
-  int* err = reinterpret_cast<int*>(ws + oNorm + 2 * sizeof(unsigned long long));
+  int* err = reinterpret_cast<int*>(ws + oErr);
   unsigned long long* dmax = reinterpret_cast<unsigned long long*>(ws + oDmax);
+  unsigned long long* norms = dmax + N;
   float* gscale = reinterpret_cast<float*>(ws + oGscale);
   float* Wt = reinterpret_cast<float*>(ws + oWt);
 
@@ -1005,14 +1017,14 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   int it = 0;
   for (it = 1; it <= max_iter && e == cudaSuccess; ++it) {
     // ---- D = inner_solve(R) ----
-    e = cudaMemsetAsync(dmax, 0, sizeof(unsigned long long) * N, s);
+    e = cudaMemsetAsync(dmax, 0, sizeof(unsigned long long) * (N + 2), s);
     if (e != cudaSuccess) break;
     const double* src = it == 1 ? B_dev : R;
     const int64_t lds = it == 1 ? ldb : ld;
     if (trsm::pairs_ok(src, lds) && trsm::pairs_ok(W, ld))
-      trsm::to_float_kernel<true><<<trsm::grid_pairs(n, k), 256, 0, s>>>(src, lds, W, ld, n, k);
+      trsm::launch_dependent(trsm::to_float_kernel<true>, trsm::grid_pairs(n, k), dim3(256), 0, s, 1, src, lds, W, ld, n, k);
     else
-      trsm::to_float_kernel<false><<<trsm::grid_pairs(n, k), 256, 0, s>>>(src, lds, W, ld, n, k);
+      trsm::launch_dependent(trsm::to_float_kernel<false>, trsm::grid_pairs(n, k), dim3(256), 0, s, 1, src, lds, W, ld, n, k);
     trsm::count_launch();
     for (int64_t i = 0; i < N && e == cudaSuccess; ++i) {
       const int64_t s0 = i * n0;
@@ -1029,12 +1041,12 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
         if (s0 % 4 == 0 && n0p % 4 == 0 && ld % 4 == 0) {
           const dim3 gv(static_cast<unsigned>((n0p / 4 + 255) / 256),
                         static_cast<unsigned>(std::min<int64_t>(k, std::max<int64_t>(1, 2432 / ((n0p / 4 + 255) / 256)))));
-          if (tc_planes == 3) trsm::pack_w_tf32_vec_kernel<3><<<gv, 256, 0, s>>>(W, ld, s0, m, k, n0p, Wt);
-          else if (tc_planes == 2) trsm::pack_w_tf32_vec_kernel<2><<<gv, 256, 0, s>>>(W, ld, s0, m, k, n0p, Wt);
-          else trsm::pack_w_tf32_vec_kernel<1><<<gv, 256, 0, s>>>(W, ld, s0, m, k, n0p, Wt);
-        } else if (tc_planes == 3) trsm::pack_w_tf32_kernel<3><<<gw, 256, 0, s>>>(W, ld, s0, m, k, n0p, Wt);
-        else if (tc_planes == 2) trsm::pack_w_tf32_kernel<2><<<gw, 256, 0, s>>>(W, ld, s0, m, k, n0p, Wt);
-        else trsm::pack_w_tf32_kernel<1><<<gw, 256, 0, s>>>(W, ld, s0, m, k, n0p, Wt);
+          if (tc_planes == 3) trsm::launch_dependent(trsm::pack_w_tf32_vec_kernel<3>, gv, dim3(256), 0, s, 1, W, ld, s0, m, k, n0p, Wt);
+          else if (tc_planes == 2) trsm::launch_dependent(trsm::pack_w_tf32_vec_kernel<2>, gv, dim3(256), 0, s, 1, W, ld, s0, m, k, n0p, Wt);
+          else trsm::launch_dependent(trsm::pack_w_tf32_vec_kernel<1>, gv, dim3(256), 0, s, 1, W, ld, s0, m, k, n0p, Wt);
+        } else if (tc_planes == 3) trsm::launch_dependent(trsm::pack_w_tf32_kernel<3>, gw, dim3(256), 0, s, 1, W, ld, s0, m, k, n0p, Wt);
+        else if (tc_planes == 2) trsm::launch_dependent(trsm::pack_w_tf32_kernel<2>, gw, dim3(256), 0, s, 1, W, ld, s0, m, k, n0p, Wt);
+        else trsm::launch_dependent(trsm::pack_w_tf32_kernel<1>, gw, dim3(256), 0, s, 1, W, ld, s0, m, k, n0p, Wt);
         trsm::count_launch();
         e = cudaGetLastError();
         if (e == cudaSuccess)
@@ -1044,12 +1056,12 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
           const dim3 gp(static_cast<unsigned>((m + 255) / 256),
                         static_cast<unsigned>(std::min<int64_t>(k, std::max<int64_t>(1, 2432 / ((m + 255) / 256)))));
           switch (mode) {
-            case 1: trsm::pack_dt_kernel<1><<<gp, 256, 0, s>>>(D, ld, s0, m, k, n0p, static_cast<float*>(Dt)); break;
+            case 1: trsm::launch_dependent(trsm::pack_dt_kernel<1>, gp, dim3(256), 0, s, 1, D, ld, s0, m, k, n0p, static_cast<float*>(Dt)); break;
             case 2:
-              trsm::pack_dt_kernel<2><<<gp, 256, 0, s>>>(D, ld, s0, m, k, n0p, static_cast<__nv_bfloat16*>(Dt));
+              trsm::launch_dependent(trsm::pack_dt_kernel<2>, gp, dim3(256), 0, s, 1, D, ld, s0, m, k, n0p, static_cast<__nv_bfloat16*>(Dt));
               break;
             default:
-              trsm::pack_dt_kernel<0><<<gp, 256, 0, s>>>(D, ld, s0, m, k, n0p, static_cast<__nv_bfloat16*>(Dt));
+              trsm::launch_dependent(trsm::pack_dt_kernel<0>, gp, dim3(256), 0, s, 1, D, ld, s0, m, k, n0p, static_cast<__nv_bfloat16*>(Dt));
               break;
           }
           trsm::count_launch();
@@ -1072,7 +1084,7 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
         if (mode == 3) {
           const dim3 gp(static_cast<unsigned>((m + 255) / 256),
                         static_cast<unsigned>(std::min<int64_t>(k, std::max<int64_t>(1, 2432 / ((m + 255) / 256)))));
-          trsm::pack_dt_f16_kernel<<<gp, 256, 0, s>>>(D, ld, s0, m, k, n0p, dmax_i, mp->panel_exp + i,
+          trsm::launch_dependent(trsm::pack_dt_f16_kernel, gp, dim3(256), 0, s, 1, D, ld, s0, m, k, n0p, dmax_i, mp->panel_exp + i,
                                                       static_cast<__half*>(Dt), gscale + i);
           trsm::count_launch();
           e = cudaGetLastError();
@@ -1088,16 +1100,15 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
       }
     }
     // ---- X += D ----
-    if (e == cudaSuccess) e = cudaMemsetAsync(norms, 0, 2 * sizeof(unsigned long long), s);
     if (e == cudaSuccess) {
       const bool vec = trsm::pairs_ok(X_dev, ldx) && trsm::pairs_ok(D, ld);
       const dim3 gc = trsm::grid_pairs(n, k);
       if (it == 1)
-        vec ? trsm::correct_kernel<true, true><<<gc, 256, 0, s>>>(X_dev, ldx, D, ld, n, k, norms)
-            : trsm::correct_kernel<false, true><<<gc, 256, 0, s>>>(X_dev, ldx, D, ld, n, k, norms);
+        vec ? trsm::launch_dependent(trsm::correct_kernel<true, true>, gc, dim3(256), 0, s, 1, X_dev, ldx, D, ld, n, k, norms)
+            : trsm::launch_dependent(trsm::correct_kernel<false, true>, gc, dim3(256), 0, s, 1, X_dev, ldx, D, ld, n, k, norms);
       else
-        vec ? trsm::correct_kernel<true, false><<<gc, 256, 0, s>>>(X_dev, ldx, D, ld, n, k, norms)
-            : trsm::correct_kernel<false, false><<<gc, 256, 0, s>>>(X_dev, ldx, D, ld, n, k, norms);
+        vec ? trsm::launch_dependent(trsm::correct_kernel<true, false>, gc, dim3(256), 0, s, 1, X_dev, ldx, D, ld, n, k, norms)
+            : trsm::launch_dependent(trsm::correct_kernel<false, false>, gc, dim3(256), 0, s, 1, X_dev, ldx, D, ld, n, k, norms);
       trsm::count_launch();
       e = cudaGetLastError();
     }

@@ -90,6 +90,8 @@ __global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restr
   constexpr int kUnits = 8 / kWarps;             // (row, chunk) pairs per CTA
   constexpr int kGroups = kWarps == 8 ? 2 : 1;   // groups of four values per lane
   __shared__ unsigned long long smax[8];
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = warp / kWarps, wu = warp % kWarps;
   const int64_t u = blockIdx.x * static_cast<int64_t>(kUnits) + unit;
@@ -484,6 +486,8 @@ __global__ void __maxnreg__(kMaxRegs)
   const int out_tiles = (a.M + 127) / 128 * a.C;
   const int items = BN / a.item_cols;  // per output tile
   if (threadIdx.x == 0) {
+    tc::prefetch_map(&mapA);
+    tc::prefetch_map(&mapB);
     for (int q = 0; q < STAGES; ++q) {
       tc::mbar_init(&full_bar[q], 1);
       tc::mbar_init(&empty_bar[q], 1);
@@ -515,11 +519,10 @@ __global__ void __maxnreg__(kMaxRegs)
   tc::tc_fence_after();
   const uint32_t tbase = tmem_base_sh;
   volatile int* abort_flag = &abort_sh;
+  grid_dependency_wait();
 
   if (warp == 0) {
     if (lane == 0) {
-      tc::prefetch_map(&mapA);
-      tc::prefetch_map(&mapB);
       int it = 0, lin;
       bool ok = true;
       for (int t = 0; ok && (lin = nth_tile(a, unit, t, total)) >= 0; ++t) {
@@ -842,28 +845,19 @@ cudaError_t launch_product(const CUtensorMap& ma, const CUtensorMap& mb, const r
   auto kern = rns::rns_product_kernel<BN, kPair>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(S::SMEM_BYTES));
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(kPair ? 2 * units : units);
-  cfg.blockDim = dim3(S::kThreads);
-  cfg.dynamicSmemBytes = S::SMEM_BYTES;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = 2;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = kPair ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, kern, ma, mb, a, err);
+  e = launch_dependent(kern, dim3(kPair ? 2 * units : units), dim3(S::kThreads), S::SMEM_BYTES, s, kPair ? 2 : 1, ma, mb, a,
+                       err);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int kWarps>
-void launch_residues(const double* src, int64_t ld, int64_t K, const RnsOperand& o, RnsClass c, bool vec,
-                     const rns::ResidueConsts& rc, cudaStream_t s) {
+cudaError_t launch_residues(const double* src, int64_t ld, int64_t K, const RnsOperand& o, RnsClass c, bool vec,
+                            const rns::ResidueConsts& rc, cudaStream_t s) {
   const int64_t units = o.rows * o.nch, per = 8 / kWarps;
-  rns::residue_rows_kernel<kWarps><<<static_cast<unsigned>((units + per - 1) / per), 256, 0, s>>>(
-      src, ld, o.rows, K, o.nch, o.kc, o.ex_ld, o.res, o.kb, o.ex, c.moduli, c.bits, o.tri ? 1 : 0, vec ? 1 : 0, rc);
+  return launch_dependent(rns::residue_rows_kernel<kWarps>, dim3(static_cast<unsigned>((units + per - 1) / per)), dim3(256),
+                          0, s, 1, src, ld, o.rows, K, o.nch, o.kc, o.ex_ld, o.res, o.kb, o.ex, c.moduli, c.bits,
+                          o.tri ? 1 : 0, vec ? 1 : 0, rc);
 }
 
 }  // namespace
@@ -922,12 +916,12 @@ cudaError_t rns_rows(const double* src, int64_t ld, int64_t K, const RnsOperand&
   // as many warps per (row, chunk) as it has groups of 128 values (the
   // padded row of a single chunk included)
   const int64_t w = std::min<int64_t>(o.kc, o.kb * rns::kStepK);
-  if (w <= 128) launch_residues<1>(src, ld, K, o, c, vec, rc, s);
-  else if (w <= 256) launch_residues<2>(src, ld, K, o, c, vec, rc, s);
-  else if (w <= 512) launch_residues<4>(src, ld, K, o, c, vec, rc, s);
-  else launch_residues<8>(src, ld, K, o, c, vec, rc, s);
+  const cudaError_t e = w <= 128   ? launch_residues<1>(src, ld, K, o, c, vec, rc, s)
+                        : w <= 256 ? launch_residues<2>(src, ld, K, o, c, vec, rc, s)
+                        : w <= 512 ? launch_residues<4>(src, ld, K, o, c, vec, rc, s)
+                                   : launch_residues<8>(src, ld, K, o, c, vec, rc, s);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 static cudaError_t transpose_and_reduce(const double* L, int64_t ldl, int64_t n, int64_t n0, const RnsOperand& o,

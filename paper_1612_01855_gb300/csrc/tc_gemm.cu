@@ -201,10 +201,10 @@ cudaError_t launch_persistent(const CUtensorMap& ma, const CUtensorMap& mb, cons
   constexpr int kTmemCols = 2 * Cfg::NG * Cfg::BN <= 128 ? 128 : 2 * Cfg::NG * Cfg::BN <= 256 ? 256 : 512;
   const int per_sm = std::max(1, std::min(static_cast<int>(kSmemPerSm / Cfg::SMEM_BYTES), 512 / kTmemCols));
   const int64_t grid = std::min<int64_t>(tiles, static_cast<int64_t>(device_sm_count()) * per_sm);
-  kern<<<static_cast<unsigned>(grid), 192, Cfg::SMEM_BYTES, s>>>(ma, mb, epi, static_cast<int>(R),
-                                                                 static_cast<int>(C), err);
+  e = launch_dependent(kern, dim3(static_cast<unsigned>(grid)), dim3(192), Cfg::SMEM_BYTES, s, 1, ma, mb, epi,
+                       static_cast<int>(R), static_cast<int>(C), err);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <bool kTf32, int BN, int STAGES>
@@ -299,14 +299,22 @@ cudaError_t gemm_split_tf32_tri(const float* A, int64_t lda, int64_t a_plane, co
   }
 }
 
+// 128 x 256 tiles that cover less than half of the SMs.
+static bool few_wide_tiles(int64_t M, int64_t N) {
+  return 2 * ((M + 127) / 128) * ((N + 255) / 256) < device_sm_count();
+}
+
 cudaError_t gemm_split_bf16(const void* A, int64_t lda, int64_t a_plane, const void* B, int64_t ldb,
                             int64_t b_plane, float* C, int64_t ldc, int64_t M, int64_t N, int64_t K, float alpha,
                             float beta, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   // a stage is 96 KB at BN = 256 (two stages); short K takes 48 KB stages
-  // at BN = 64 so that two CTAs share an SM
+  // at BN = 64 so that two CTAs share an SM, and longer K four of them where
+  // wide tiles would leave SMs idle
   const int kb = static_cast<int>((K * 2 + 127) / 128);
   if (kb <= 8) return split_gemm<64, 2>(A, lda, a_plane, B, ldb, b_plane, C, ldc, M, N, K, alpha, beta, err, s);
+  if (few_wide_tiles(M, N))
+    return split_gemm<64, 4>(A, lda, a_plane, B, ldb, b_plane, C, ldc, M, N, K, alpha, beta, err, s);
   return split_gemm<256, 2>(A, lda, a_plane, B, ldb, b_plane, C, ldc, M, N, K, alpha, beta, err, s);
 }
 
@@ -317,6 +325,8 @@ cudaError_t gemm_split_f16(const void* A, int64_t lda, int64_t a_plane, const vo
   const int kb = static_cast<int>((K * 2 + 127) / 128);
   if (kb <= 8)
     return split_gemm<64, 2, true>(A, lda, a_plane, B, ldb, b_plane, C, ldc, M, N, K, alpha, beta, err, s, scale);
+  if (few_wide_tiles(M, N))
+    return split_gemm<64, 4, true>(A, lda, a_plane, B, ldb, b_plane, C, ldc, M, N, K, alpha, beta, err, s, scale);
   return split_gemm<256, 2, true>(A, lda, a_plane, B, ldb, b_plane, C, ldc, M, N, K, alpha, beta, err, s, scale);
 }
 
@@ -331,6 +341,9 @@ cudaError_t gemm_lowp(bool tf32, const void* A, int64_t lda, const void* B, int6
   if (kb <= 8)
     return tf32 ? plain_gemm<true, 128, 2>(A, lda, B, ldb, C, M, N, K, ldc, alpha, beta, err, s)
                 : plain_gemm<false, 128, 2>(A, lda, B, ldb, C, M, N, K, ldc, alpha, beta, err, s);
+  if (few_wide_tiles(M, N))
+    return tf32 ? plain_gemm<true, 64, 8>(A, lda, B, ldb, C, M, N, K, ldc, alpha, beta, err, s)
+                : plain_gemm<false, 64, 8>(A, lda, B, ldb, C, M, N, K, ldc, alpha, beta, err, s);
   // 128 x 256 tiles: 48 KB a stage, a quarter less operand traffic per flop
   // than 128 x 128 (measured at 8192^3: bf16 979 -> 1500, tf32 521 -> 817
   // TFLOP/s)

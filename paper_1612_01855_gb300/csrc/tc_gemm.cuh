@@ -15,6 +15,7 @@
 // hold an exact integer sum over one chunk (used by the sliced FP64
 // emulation).  A plain GEMM is NSA = NSB = NG = 1 and a single chunk.
 #pragma once
+#include "internal.h"
 #include "tc_engine.cuh"
 
 namespace trsm {
@@ -214,6 +215,8 @@ __global__ void __launch_bounds__(192, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = R * C;
   if (threadIdx.x == 0) {
+    prefetch_map(&mapA);
+    prefetch_map(&mapB);
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
@@ -234,11 +237,10 @@ __global__ void __launch_bounds__(192, 1)
   tc_fence_after();
   const uint32_t tbase = tmem_base_sh;
   volatile int* abort_flag = &abort_sh;
+  grid_dependency_wait();
 
   if (warp == 0) {
     if (lane == 0) {
-      prefetch_map(&mapA);
-      prefetch_map(&mapB);
       int it = 0;  // stage uses so far, across tiles
       for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
         int tm = 0, tn = 0, kb0 = 0, kb1 = 0, chunk = 1;
