@@ -263,6 +263,17 @@ constexpr int kSysMaxCW = 32;  // widest column chunk of a unit
 // operands staged by cp.async into two buffers instead of through
 // registers, 1.60 -> 2.05 ms at five CTAs per SM; L~_ll alone copied by
 // cp.async behind the product, 1.74 ms.)
+// The unit kernel is bound by the shared-memory and L1 data path (91 % of
+// its cycles while an SM is active, the FMA pipe 35 %): each 4 x 4 output
+// tile of a thread loads 8 registers for 16 multiply-adds.  So its stores
+// avoid bank conflicts: the X operand is staged 8 rows x 4 columns to a warp
+// (banks 36 kk + col all different; a row per lane conflicts four ways), W
+// and X_b0 are stored four columns at a time.  4096 mixed systems, a
+// graph replay: the conflicting stores 1.332 ms, these 1.303 ms.  (Measured
+// no faster: a warp forming the whole 64 x 32 tile over a quarter of K, 8 x 8
+// outputs to a lane, operands by cp.async, which needs a third less of that
+// data path but leaves room for 16 warps on an SM instead of 24: 1.361 ms;
+// with the next step's first slice fetched ahead, 1.389 ms.)
 struct SysSmem {
   union {
     float inv[64][68];  // inv[col][row]: L~_ll, zeros above the diagonal (rows 16-byte aligned)
@@ -425,6 +436,16 @@ struct UnitSys {
   int N;
 };
 
+template <int CPT>
+__device__ __forceinline__ void store_row(float* p, const float (&v)[CPT]) {
+  if constexpr (CPT == 4)
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else if constexpr (CPT == 2)
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  else
+    *p = v[0];
+}
+
 // TM (4 or 8) consecutive floats of a 16-byte aligned shared-memory row.
 template <int TM>
 __device__ __forceinline__ void load_rows(const float* p, float (&v)[TM]) {
@@ -454,10 +475,10 @@ __device__ void sys_unit(const UnitSys& a, int c0, SysSmem& sm) {
   const int tid = threadIdx.x, ty = tid / TX, tx = tid % TX;
   const int nc = static_cast<int>(imin64(CW, a.k - c0));
   // staging roles: A value it is L(s0 + arow, t0 + akk + 2 it), B value it
-  // is X(t0 + bkk, c0 + bcol + 4 it) (CW = 32: 4 it spans the 32 columns)
+  // is X(t0 + bkk, c0 + bcol + 4 it), a warp on 8 rows x 4 columns
   const int arow = tid & 63, akk = tid >> 6;
-  const int bkk = tid & 31, bcol = tid >> 5;
-  constexpr int kBColStep = kSysThreads / 32;
+  const int bkk = 8 * (tid >> 5) + (tid & 7), bcol = (tid >> 3) & 3;
+  constexpr int kBColStep = 4;
   const int64_t astep = 2 * a.ldl, bstep = kBColStep * a.ldx;
   bool bok[NB];
 #pragma unroll
@@ -532,13 +553,13 @@ __device__ void sys_unit(const UnitSys& a, int c0, SysSmem& sm) {
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int row = ty * TM + i;
+      float wv[CPT];
 #pragma unroll
       for (int j = 0; j < CPT; ++j) {
         const int col = tx * CPT + j;
-        sm.w[row][col] = (row < m && col < nc)
-                             ? a.B[static_cast<int64_t>(c0 + col) * a.ldb + s0 + row] - acc[i][j]
-                             : 0.f;
+        wv[j] = (row < m && col < nc) ? a.B[static_cast<int64_t>(c0 + col) * a.ldb + s0 + row] - acc[i][j] : 0.f;
       }
+      store_row<CPT>(&sm.w[row][tx * CPT], wv);
     }
     __syncthreads();
     // X_l = L~_ll W_l.  L~_ll is lower triangular and warp w holds rows
@@ -610,8 +631,8 @@ __device__ void sys_unit_pair(const UnitSys& a, int c0, SysSmem& sm) {
   const int tid = threadIdx.x, ty = tid / TX, tx = tid % TX;
   const int nc = static_cast<int>(imin64(CW, a.k - c0));
   const int arow = tid & 63, akk = tid >> 6;
-  const int bkk = tid & 31, bcol = tid >> 5;
-  constexpr int kBColStep = kSysThreads / 32;
+  const int bkk = 8 * (tid >> 5) + (tid & 7), bcol = (tid >> 3) & 3;
+  constexpr int kBColStep = 4;
   const int64_t astep = 2 * a.ldl, bstep = kBColStep * a.ldx;
   bool bok[NB];
 #pragma unroll
@@ -695,13 +716,13 @@ __device__ void sys_unit_pair(const UnitSys& a, int c0, SysSmem& sm) {
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int row = ty * TM + i;
+      float wv[CPT];
 #pragma unroll
       for (int j = 0; j < CPT; ++j) {
         const int col = tx * CPT + j;
-        sm.w[row][col] = (row < m && col < nc)
-                             ? a.B[static_cast<int64_t>(c0 + col) * a.ldb + s0 + row] - acc[i][j]
-                             : 0.f;
+        wv[j] = (row < m && col < nc) ? a.B[static_cast<int64_t>(c0 + col) * a.ldb + s0 + row] - acc[i][j] : 0.f;
       }
+      store_row<CPT>(&sm.w[row][tx * CPT], wv);
     }
     __syncthreads();
     const int r0 = 2 * ty;
@@ -714,11 +735,12 @@ __device__ void sys_unit_pair(const UnitSys& a, int c0, SysSmem& sm) {
     half_mma<CW>(sm.p.i11, &sm.w[0][0], LDW, min((m0 + 7) & ~7, warp_end), ty, tx, x);
     __syncthreads();  // every read of W_top done before it is overwritten by X_b0
 #pragma unroll
+    for (int i = 0; i < 2; ++i) store_row<CPT>(&sm.w[r0 + i][tx * CPT], x[i]);
+#pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < CPT; ++j) {
         const int row = r0 + i, col = tx * CPT + j;
-        sm.w[row][col] = x[i][j];
         if (row < m0 && col < nc) a.X[static_cast<int64_t>(c0 + col) * a.ldx + s0 + row] = x[i][j];
       }
     __syncthreads();
@@ -730,9 +752,13 @@ __device__ void sys_unit_pair(const UnitSys& a, int c0, SysSmem& sm) {
         for (int j = 0; j < CPT; ++j) x[i][j] = 0.f;
       half_mma<CW>(sm.p.l21, &sm.w[0][0], LDW, (m0 + 7) & ~7, ty, tx, x);
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < 2; ++i) {
+        float wv[CPT];
+        load_row<CPT>(&sm.w[32 + r0 + i][tx * CPT], wv);
 #pragma unroll
-        for (int j = 0; j < CPT; ++j) sm.w[32 + r0 + i][tx * CPT + j] -= x[i][j];
+        for (int j = 0; j < CPT; ++j) wv[j] -= x[i][j];
+        store_row<CPT>(&sm.w[32 + r0 + i][tx * CPT], wv);
+      }
       __syncthreads();
       // X_b1 = L~_b1 W_bot
 #pragma unroll
