@@ -39,6 +39,24 @@ std::vector<trsm::DiagBlock> diag_blocks(int64_t n, int64_t n0, int64_t ld, bool
   return v;
 }
 
+// Memory of L~.  Small plans take it from a pool instead of
+// mapping and unmapping fresh memory (cudaMalloc, cudaFree): at n = 512 a
+// plan and its destruction took 250 and 105 us, 90 and 4 us so, with no wait
+// for the descriptors' copy.  The pool keeps at most what the small
+// plans alive at one time needed, and gives it back like any workspace.  A
+// capturing stream, on which a plan cannot be made, fails as it does with
+// cudaMalloc.
+constexpr size_t kPoolPlanBytes = (size_t)32 << 20;
+cudaError_t alloc_lt(double** p, size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+  if (bytes <= kPoolPlanBytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    trsm::keep_small_block();
+    return trsm::plan_alloc((void**)p, bytes, s);
+  }
+  cudaGetLastError();
+  return cudaMalloc((void**)p, bytes);
+}
+
 // Inverts the listed blocks and reports a singular pivot.  Synchronous.
 int invert_and_check(double* A, int64_t ld, const std::vector<trsm::DiagBlock>& blocks,
                      cudaStream_t s) {
@@ -47,11 +65,13 @@ int invert_and_check(double* A, int64_t ld, const std::vector<trsm::DiagBlock>& 
   if (e != cudaSuccess) return from_cuda(e);
   unsigned long long h_sing = ULLONG_MAX;
   e = cudaMemsetAsync(sing, 0xFF, sizeof(unsigned long long), s);
-  if (e == cudaSuccess) e = trsm::invert_diag_blocks(A, ld, blocks, sing, s);
+  std::vector<unsigned char> desc;  // read by a copy on s: lives until s has been waited for
+  if (e == cudaSuccess) e = trsm::invert_diag_blocks(A, ld, blocks, sing, desc, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(&h_sing, sing, sizeof(h_sing), cudaMemcpyDeviceToHost, s);
   trsm::ws_free(sing, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return from_cuda(e);
   if (h_sing != ULLONG_MAX) {
     t_singular = (int64_t)h_sing;
@@ -159,7 +179,7 @@ int trsm_plan(const double* L_dev, int64_t n, int64_t ldl, int64_t n0, void* str
   h->N = (n + n0 - 1) / n0;
   h->ldt = align4(n);
   cudaGetDevice(&h->device);
-  cudaError_t e = cudaMalloc((void**)&h->Lt, sizeof(double) * (size_t)h->ldt * (size_t)n);
+  cudaError_t e = alloc_lt(&h->Lt, sizeof(double) * (size_t)h->ldt * (size_t)n, s);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), s);
   if (e == cudaSuccess) e = trsm::copy_lower(L_dev, ldl, h->Lt, h->ldt, n, s);
@@ -333,9 +353,11 @@ void trsm_destroy(trsm_handle_t h) {
   int cur = 0;
   cudaGetDevice(&cur);
   if (cur != h->device) cudaSetDevice(h->device);
-  // cudaFree waits for the device work that may still use the memory.
-  if (h->Lt) cudaFree(h->Lt);
+  // The cudaFree of the status word, which is cudaMalloc's, waits for the
+  // device work that may still use the plan; that of L~ need not wait (where
+  // it is the pool's) or waits again.
   if (h->status) cudaFree(h->status);
+  if (h->Lt) cudaFree(h->Lt);
   trsm::mixed_release(h);
   trsm::sliced_release(h);
   if (cur != h->device) cudaSetDevice(cur);

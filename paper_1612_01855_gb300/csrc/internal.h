@@ -48,9 +48,11 @@ struct DiagBlock {
 // by recursive triangular inversion; the strict upper triangle of each block
 // must hold zeros on entry.  The smallest row index with a zero or non-finite
 // pivot is folded (atomic min) into *sing_dev.  Asynchronous on `s`;
-// allocates its scratch stream-ordered.  Returns a cudaError_t.
+// allocates its scratch stream-ordered.  `host` takes the descriptors that a
+// copy on `s` reads: the caller keeps it until `s` has been waited for.
+// Returns a cudaError_t.
 cudaError_t invert_diag_blocks(double* A, int64_t ld, const std::vector<DiagBlock>& blocks,
-                               unsigned long long* sing_dev, cudaStream_t s);
+                               unsigned long long* sing_dev, std::vector<unsigned char>& host, cudaStream_t s);
 
 // Lt(i, j) = (i >= j) ? L(i, j) : 0 for an n x n matrix.
 cudaError_t copy_lower(const double* L, int64_t ldl, double* Lt, int64_t ldt, int64_t n,
@@ -102,6 +104,10 @@ int plan_device(trsm_handle_t h);
 // mapping again at each call (about 1 ms per GB).  trsm_workspace_trim
 // returns the pool's idle memory (pool.cu).
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
+// The same from a pool for plans, to be freed by cudaFree once its last use
+// is over; keep_small_block makes cudaMalloc and cudaFree of single words cheap.
+cudaError_t plan_alloc(void** p, size_t bytes, cudaStream_t s);
+void keep_small_block();
 cudaError_t ws_free(void* p, cudaStream_t s);
 template <class T>
 cudaError_t ws_alloc(T** p, size_t bytes, cudaStream_t s) {

@@ -15,7 +15,9 @@
 //     on separate streams are never ordered behind one another by their
 //     scratch.  A block whose free has completed is reused on any stream.
 // trsm_workspace_trim hands the idle memory back; an allocation that fails
-// trims the pool and retries once.
+// trims the pools and retries once.
+// Small plans' L~ comes from a second pool with the same settings, so that a
+// plan's block does not sit in the middle of the workspaces' memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
@@ -56,15 +58,38 @@ constexpr int kMaxDevices = 64;
 struct DevicePool {
   unsigned long long ctx_id = 0;  // context the pool was made in (0: none yet)
   cudaMemPool_t pool = nullptr;
+  cudaMemPool_t plans = nullptr;
+  bool anchored = false;  // keep_small_block has run in this context
 };
 
 std::mutex g_pool_mutex;
 DevicePool g_pools[kMaxDevices];
 
-// The pool of the current device, made at its first use in the current
-// context.  A pool of an earlier context (before a cudaDeviceReset) went
-// away with that context and is not destroyed again.
-cudaError_t current_pool(cudaMemPool_t* out) {
+cudaError_t make_pool(int dev, cudaMemPool_t* out) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t p = nullptr;
+  cudaError_t e = cudaMemPoolCreate(&p, &props);
+  if (e != cudaSuccess) return e;
+  unsigned long long keep = ~0ull;
+  int no = 0;
+  e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+  if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p, cudaMemPoolReuseAllowInternalDependencies, &no);
+  if (e != cudaSuccess) {
+    cudaMemPoolDestroy(p);
+    return e;
+  }
+  *out = p;
+  return cudaSuccess;
+}
+
+// The pools of the current device, made at their first use in the current
+// context.  Those of an earlier context (before a cudaDeviceReset) went away
+// with that context and are not destroyed again.
+cudaError_t current_pools(DevicePool* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -78,43 +103,61 @@ cudaError_t current_pool(cudaMemPool_t* out) {
   std::lock_guard<std::mutex> lock(g_pool_mutex);
   DevicePool& d = g_pools[dev];
   if (d.pool == nullptr || id == 0 || id != d.ctx_id) {
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.handleTypes = cudaMemHandleTypeNone;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t p = nullptr;
-    e = cudaMemPoolCreate(&p, &props);
+    DevicePool fresh;
+    fresh.ctx_id = id;
+    e = make_pool(dev, &fresh.pool);
     if (e != cudaSuccess) return e;
-    unsigned long long keep = ~0ull;
-    int no = 0;
-    e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p, cudaMemPoolReuseAllowInternalDependencies, &no);
+    e = make_pool(dev, &fresh.plans);
     if (e != cudaSuccess) {
-      cudaMemPoolDestroy(p);
+      cudaMemPoolDestroy(fresh.pool);
       return e;
     }
-    d.pool = p;
-    d.ctx_id = id;
+    d = fresh;
   }
-  *out = d.pool;
+  *out = d;
   return cudaSuccess;
+}
+
+cudaError_t alloc_from(cudaMemPool_t DevicePool::*which, void** p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  DevicePool d;
+  cudaError_t e = current_pools(&d);
+  if (e != cudaSuccess) return e;
+  e = cudaMallocFromPoolAsync(p, bytes, d.*which, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaMemPoolTrimTo(d.pool, 0);
+    cudaMemPoolTrimTo(d.plans, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, d.*which, s);
+  }
+  return e;
 }
 
 }  // namespace
 
-cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s) {
-  *p = nullptr;
-  cudaMemPool_t pool = nullptr;
-  cudaError_t e = current_pool(&pool);
-  if (e != cudaSuccess) return e;
-  e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-  if (e == cudaErrorMemoryAllocation) {
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s) { return alloc_from(&DevicePool::pool, p, bytes, s); }
+
+cudaError_t plan_alloc(void** p, size_t bytes, cudaStream_t s) { return alloc_from(&DevicePool::plans, p, bytes, s); }
+
+// cudaMalloc cuts small allocations from blocks of a few MB, which cudaFree
+// unmaps when the last one in them goes.  A plan's status word would
+// otherwise map and unmap such a block each time: a 64 x 64 plan took 187 us
+// to make and 62 us to destroy, 88 and 4 us with the block kept.  One word
+// per device and context is never freed.
+void keep_small_block() {
+  DevicePool now;
+  if (current_pools(&now) != cudaSuccess || now.anchored) return;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  DevicePool& d = g_pools[dev];
+  if (d.anchored || d.pool != now.pool) return;
+  void* word = nullptr;
+  if (cudaMalloc(&word, sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
-    cudaMemPoolTrimTo(pool, 0);
-    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    return;
   }
-  return e;
+  d.anchored = true;
 }
 
 cudaError_t ws_free(void* p, cudaStream_t s) { return p ? cudaFreeAsync(p, s) : cudaSuccess; }
@@ -127,14 +170,19 @@ extern "C" int trsm_workspace_trim(size_t keep_bytes) {
     cudaGetLastError();
     return TRSM_ECUDA;
   }
-  cudaMemPool_t pool = nullptr;
+  trsm::DevicePool now;
   {
     std::lock_guard<std::mutex> lock(trsm::g_pool_mutex);
     const trsm::DevicePool& d = trsm::g_pools[dev];
     if (d.pool == nullptr || d.ctx_id != trsm::current_context_id()) return TRSM_SUCCESS;  // nothing held
-    pool = d.pool;
+    now = d;
   }
-  if (cudaMemPoolTrimTo(pool, keep_bytes) != cudaSuccess) {
+  // keep_bytes in all: the workspaces' pool first, the plans' what is left
+  unsigned long long held = 0;
+  cudaError_t e = cudaMemPoolTrimTo(now.pool, keep_bytes);
+  if (e == cudaSuccess) e = cudaMemPoolGetAttribute(now.pool, cudaMemPoolAttrReservedMemCurrent, &held);
+  if (e == cudaSuccess) e = cudaMemPoolTrimTo(now.plans, held < keep_bytes ? keep_bytes - held : 0);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return TRSM_ECUDA;
   }
@@ -150,10 +198,11 @@ extern "C" size_t trsm_workspace_reserved_bytes(void) {
   std::lock_guard<std::mutex> lock(trsm::g_pool_mutex);
   const trsm::DevicePool& d = trsm::g_pools[dev];
   if (d.pool == nullptr || d.ctx_id != trsm::current_context_id()) return 0;
-  unsigned long long v = 0;
-  if (cudaMemPoolGetAttribute(d.pool, cudaMemPoolAttrReservedMemCurrent, &v) != cudaSuccess) {
+  unsigned long long v = 0, w = 0;
+  if (cudaMemPoolGetAttribute(d.pool, cudaMemPoolAttrReservedMemCurrent, &v) != cudaSuccess ||
+      cudaMemPoolGetAttribute(d.plans, cudaMemPoolAttrReservedMemCurrent, &w) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  return static_cast<size_t>(v);
+  return static_cast<size_t>(v + w);
 }

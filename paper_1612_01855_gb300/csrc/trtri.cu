@@ -288,7 +288,7 @@ struct TreeBuilder {
 }  // namespace
 
 cudaError_t invert_diag_blocks(double* A, int64_t ld, const std::vector<DiagBlock>& blocks,
-                               unsigned long long* sing_dev, cudaStream_t s) {
+                               unsigned long long* sing_dev, std::vector<unsigned char>& host, cudaStream_t s) {
   TreeBuilder tb;
   tb.ld = ld;
   for (const DiagBlock& b : blocks)
@@ -310,7 +310,7 @@ cudaError_t invert_diag_blocks(double* A, int64_t ld, const std::vector<DiagBloc
   }
   const size_t leaf_bytes = tb.leaves.size() * sizeof(LeafDesc);
   const size_t node_bytes = node_total * sizeof(NodeDesc);
-  std::vector<unsigned char> host(leaf_bytes + node_bytes);
+  host.resize(leaf_bytes + node_bytes);
   memcpy(host.data(), tb.leaves.data(), leaf_bytes);
   size_t pos = leaf_bytes;
   for (auto& lvl : tb.by_height) {
@@ -329,11 +329,6 @@ cudaError_t invert_diag_blocks(double* A, int64_t ld, const std::vector<DiagBloc
     }
   }
   e = cudaMemcpyAsync(desc, host.data(), host.size(), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) {
-    // The copy above reads pageable host memory; make sure it has been
-    // consumed before `host` goes out of scope.
-    e = cudaStreamSynchronize(s);
-  }
   if (e == cudaSuccess) {
     const LeafDesc* d_leaves = (const LeafDesc*)desc;
     leaf_inverse_kernel<<<(unsigned)tb.leaves.size(), NTHREADS, 0, s>>>(A, ld, d_leaves, sing_dev);
