@@ -37,9 +37,8 @@ SWEEP_N0 = [64, 128, 256, 512, 1024, None]  # None = n (full inversion)
 SCHEDULE_NAMES = ("dag", "right-looking", "recursive", "sliced")
 # Block sizes of the sliced schedule (FP64-class products on the tensor
 # cores): longer blocks mean longer, more efficient tensor-core products
-# (measured, ms: 16384x256 9.7 / 7.2 / 5.8 at n0 = 256 / 512 / 1024;
-# 8192x8192 26.0 / 22.0 / 20.0 at 512 / 1024 / 2048; 2048x131072 32.4 /
-# 29.7 / 30.3 at 512 / 1024 / 2048)
+# (measured, ms: 16384x256 5.3 / 1.28 at n0 = 256 / 2048; 8192x8192
+# 10.9 / 6.1 at 512 / 2048; 2048x131072 8.2 at 2048)
 SLICED_N0 = {(16384, 256): 2048, (8192, 8192): 2048, (2048, 131072): 2048}
 SLICED_PREC_N0 = 2048  # block order of the sliced schedule's precision-configuration row
 # Block size of the mixed-precision figure (n = 16384, k = 4096).  Larger

@@ -1,7 +1,7 @@
 // Device memory of the library's per-call workspaces.
 //
 // Every solve, plan and batch run takes its scratch (the working copy of B,
-// digit planes, dependency counters, partial sums) from a stream-ordered
+// residues, dependency counters, partial sums) from a stream-ordered
 // memory pool owned by the library, one per device and CUDA context.  The
 // pool differs from the device's default pool in two settings:
 //   - its release threshold is unbounded: memory freed by a call stays
