@@ -39,13 +39,14 @@ std::vector<trsm::DiagBlock> diag_blocks(int64_t n, int64_t n0, int64_t ld, bool
   return v;
 }
 
-// Memory of L~.  Small plans take it from a pool instead of
-// mapping and unmapping fresh memory (cudaMalloc, cudaFree): at n = 512 a
-// plan and its destruction took 250 and 105 us, 90 and 4 us so, with no wait
-// for the descriptors' copy.  The pool keeps at most what the small
-// plans alive at one time needed, and gives it back like any workspace.  A
-// capturing stream, on which a plan cannot be made, fails as it does with
-// cudaMalloc.
+// Memory of L~.  Small plans take it from a pool instead of mapping and
+// unmapping fresh memory (cudaMalloc, cudaFree): at n = 512 a plan and its
+// destruction took 250 and 105 us, 90 and 4 us so, with no wait for the
+// descriptors' copy.  The line lies where that mapping stops mattering beside
+// the solves a plan is made for (134 MB, n = 4096: 112 of 1200 us for a plan
+// and a solve of 16 columns go into its destruction) and bounds what idles in
+// the pool (pool.cu).  A capturing stream, on which a plan cannot be made,
+// fails as it does with cudaMalloc.
 constexpr size_t kPoolPlanBytes = (size_t)32 << 20;
 cudaError_t alloc_lt(double** p, size_t bytes, cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
@@ -179,8 +180,8 @@ int trsm_plan(const double* L_dev, int64_t n, int64_t ldl, int64_t n0, void* str
   h->N = (n + n0 - 1) / n0;
   h->ldt = align4(n);
   cudaGetDevice(&h->device);
-  cudaError_t e = alloc_lt(&h->Lt, sizeof(double) * (size_t)h->ldt * (size_t)n, s);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->status, sizeof(int));
+  cudaError_t e = cudaMalloc((void**)&h->status, sizeof(int));
+  if (e == cudaSuccess) e = alloc_lt(&h->Lt, sizeof(double) * (size_t)h->ldt * (size_t)n, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), s);
   if (e == cudaSuccess) e = trsm::copy_lower(L_dev, ldl, h->Lt, h->ldt, n, s);
   int rc = from_cuda(e);

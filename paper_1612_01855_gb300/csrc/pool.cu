@@ -16,8 +16,10 @@
 //     scratch.  A block whose free has completed is reused on any stream.
 // trsm_workspace_trim hands the idle memory back; an allocation that fails
 // trims the pools and retries once.
-// Small plans' L~ comes from a second pool with the same settings, so that a
-// plan's block does not sit in the middle of the workspaces' memory.
+// Small plans' L~ comes from a second pool, so that a plan's block does not
+// sit in the middle of the workspaces' memory.  Destroyed plans leave at most
+// kKeepPlans of it mapped: a program that held thousands of plans gets the
+// rest back at its next synchronisation.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
@@ -54,6 +56,7 @@ unsigned long long current_context_id() {
 namespace {
 
 constexpr int kMaxDevices = 64;
+constexpr unsigned long long kKeepPlans = 256ull << 20;
 
 struct DevicePool {
   unsigned long long ctx_id = 0;  // context the pool was made in (0: none yet)
@@ -65,7 +68,7 @@ struct DevicePool {
 std::mutex g_pool_mutex;
 DevicePool g_pools[kMaxDevices];
 
-cudaError_t make_pool(int dev, cudaMemPool_t* out) {
+cudaError_t make_pool(int dev, unsigned long long keep, cudaMemPool_t* out) {
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.handleTypes = cudaMemHandleTypeNone;
@@ -74,7 +77,6 @@ cudaError_t make_pool(int dev, cudaMemPool_t* out) {
   cudaMemPool_t p = nullptr;
   cudaError_t e = cudaMemPoolCreate(&p, &props);
   if (e != cudaSuccess) return e;
-  unsigned long long keep = ~0ull;
   int no = 0;
   e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
   if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p, cudaMemPoolReuseAllowInternalDependencies, &no);
@@ -105,9 +107,9 @@ cudaError_t current_pools(DevicePool* out) {
   if (d.pool == nullptr || id == 0 || id != d.ctx_id) {
     DevicePool fresh;
     fresh.ctx_id = id;
-    e = make_pool(dev, &fresh.pool);
+    e = make_pool(dev, ~0ull, &fresh.pool);
     if (e != cudaSuccess) return e;
-    e = make_pool(dev, &fresh.plans);
+    e = make_pool(dev, kKeepPlans, &fresh.plans);
     if (e != cudaSuccess) {
       cudaMemPoolDestroy(fresh.pool);
       return e;
