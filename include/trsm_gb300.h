@@ -58,7 +58,8 @@ extern "C" {
 /* The sliced residuals run on the bf16 tensor cores in integer arithmetic: L
  * to 48 bits of each (row, 2048-wide chunk) maximum, X to 42 bits of each
  * (column, chunk) maximum in the seven-plane class, 48 in the eight-plane
- * class (35 in the classes of five and six), exact products. */
+ * class (35 in the classes of five and six), products to 2^-49 of the
+ * maxima's, exactly for factors of up to nine 6-bit digits a pair. */
 #define TRSM_RESIDUAL_SLICED 0   /* FP64-class: the seven-plane class */
 #define TRSM_RESIDUAL_FP64 1     /* FP64 fused multiply-add                                */
 #define TRSM_RESIDUAL_SLICED8 2  /* the eight-plane class: ~2^-50 instead of ~2^-45 */
@@ -142,11 +143,12 @@ int trsm_solve(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, dou
  *                             bits below a power-of-two exponent per row (per
  *                             row and block column for L), its residues
  *                             modulo 15 small primes and prime powers are
- *                             multiplied with exact FP32 sums, and the exact
- *                             integer products are put together from their
- *                             residues and applied in FP64.  Each product
- *                             carries about 2^-49 of |A| |B| (an FP64-class
- *                             result, not FP64 rounding).
+ *                             multiplied with exact FP32 sums, and the integer
+ *                             products are put together from their residues
+ *                             and applied in FP64.  Each product carries
+ *                             about 2^-49 of |A| |B| (an FP64-class result,
+ *                             not FP64 rounding); factors of up to nine
+ *                             6-bit digits a pair give exact products.
  *                             Needs trsm_plan_sliced on the plan first
  *                             (else TRSM_EINVAL) and k <= 5242800; X_dev
  *                             may equal B_dev with ldx == ldb.

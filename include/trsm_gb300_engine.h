@@ -34,8 +34,9 @@ int trsm_tc_gemm_selftest(int mode, const void* A_dev, const void* B_dev, float*
  * strictly lower L and X are rounded to integers of 48 bits and, for planes
  * = 5 .. 8, of 35, 35, 42 or 48 bits per (row, 2048-wide chunk of K) with a
  * power-of-two exponent each; their residues modulo 13, 13, 14 or 15 moduli
- * are multiplied with exact FP32 sums, and the chunk's exact integer product
- * is put together from them and applied in FP64 (after Ozaki, Uchino &
+ * are multiplied with exact FP32 sums, and the chunk's integer product is put
+ * together from them (to 3.2 2^-64 of the moduli's product, exactly for
+ * factors of up to nine 6-bit digits a pair) and applied in FP64 (after Ozaki, Uchino &
  * Imamura 2025); the diagonal of L is applied in FP64.  Relative error about
  * 2^-45 (7 planes) or 2^-50 (8 planes) of (|B| + |L| |X|), about 2^-38 with
  * 5 or 6.

@@ -994,6 +994,7 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   void* Dt = ws + oDt;
   trsm::RnsOperand Xs = trsm::rns_operand_view(ws + oXs, k, n);
   const trsm::RnsScratch scratch = trsm::rns_scratch_view(ws + oPart, n, k);
+  Xs.zmax = scratch.zmax;
   int* err = reinterpret_cast<int*>(ws + oErr);
   unsigned long long* dmax = reinterpret_cast<unsigned long long*>(ws + oDmax);
   unsigned long long* norms = dmax + N;
@@ -1219,8 +1220,9 @@ extern "C" int trsm_residual_plan(trsm_handle_t h, const double* X_dev, int64_t 
   unsigned char* buf = nullptr;
   cudaError_t e = trsm::ws_alloc(reinterpret_cast<void**>(&buf), xb + pb, s);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TRSM_ENOMEM : TRSM_ECUDA;
-  const trsm::RnsOperand Xs = trsm::rns_operand_view(buf, k, n);
+  trsm::RnsOperand Xs = trsm::rns_operand_view(buf, k, n);
   const trsm::RnsScratch sc = trsm::rns_scratch_view(buf + xb, n, k);
+  Xs.zmax = sc.zmax;
   e = trsm::rns_scratch_clear(sc, s);
   if (e == cudaSuccess) e = trsm::rns_rows(X_dev, ldx, n, Xs, trsm::rns_class(planes), s);
   if (e == cudaSuccess)

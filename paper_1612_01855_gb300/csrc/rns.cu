@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "internal.h"
 #include "rns.h"
@@ -26,6 +27,10 @@ constexpr int kMaxResidue = 90;
 static_assert(kChunk * kMaxResidue * kMaxResidue < (1 << 24), "a chunk's sums must be exact in FP32");
 
 constexpr int kNonFinite = INT16_MAX;  // exponent of a (row, chunk) that holds an infinity or a NaN
+// 6-bit digits of zeros that end the integers of two factors, together, from
+// which their product is put together exactly: nine digits are left of 48 and
+// 48 bits.
+constexpr int kExactDigits = 7;
 constexpr float kRound = 12582912.f;   // 1.5 * 2^23: x + kRound - kRound rounds |x| < 2^22 to an integer
 constexpr int kStepK = 64;             // one 128-byte swizzled row of bf16
 
@@ -80,16 +85,21 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
 // bytes) per modulus.  The chunk's values stay in registers between the
 // maximum and the conversion (at most 2048 / (32 kWarps) = 8 a lane), so
 // they are read once.  Bound by HBM: 8 bytes read and 2 bytes per modulus
-// written per value.
+// written per value.  zeros[r ex_stride + c]: the 6-bit digits (0 to 7) that
+// end every integer of the (row, chunk) in zeros; their maximum is folded into
+// *zmax.  A value with one of its lowest 11 bits set leaves none, which settles
+// nearly every warp with one vote.
 template <int kWarps>
 __global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restrict__ src, int64_t ld, int64_t rows,
                                                            int64_t K, int64_t nch, int64_t kc, int64_t ex_stride,
                                                            __nv_bfloat16* __restrict__ dst, int64_t kb,
-                                                           int16_t* __restrict__ ex, int moduli, int bits, int tri, int vec,
+                                                           int16_t* __restrict__ ex, int8_t* __restrict__ zeros,
+                                                           int* zmax, int moduli, int bits, int tri, int vec,
                                                            const __grid_constant__ ResidueConsts rc) {
   constexpr int kUnits = 8 / kWarps;             // (row, chunk) pairs per CTA
   constexpr int kGroups = kWarps == 8 ? 2 : 1;   // groups of four values per lane
   __shared__ unsigned long long smax[8];
+  __shared__ int slow[8];
   grid_launch_dependents();
   grid_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -102,6 +112,7 @@ __global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restr
   const double* p = src + r * ld;
   double v[kGroups][4];
   unsigned long long mb = 0;
+  uint32_t tail = 0;
 #pragma unroll
   for (int g = 0; g < kGroups; ++g) {
     const int64_t k = k0 + 4 * (g * 32 * kWarps + wu * 32 + lane);
@@ -119,6 +130,7 @@ __global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restr
     for (int q = 0; q < 4; ++q) {
       const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v[g][q])) & ~(1ull << 63);
       mb = b > mb ? b : mb;
+      tail |= static_cast<uint32_t>(b);
     }
   }
 #pragma unroll
@@ -126,8 +138,20 @@ __global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restr
     const unsigned long long b = __shfl_xor_sync(0xffffffffu, mb, o);
     mb = b > mb ? b : mb;
   }
+  // the lowest bit that is set in any value of the warp: 2^(low - 1075)
+  int low = INT_MIN;
+  if (!__any_sync(0xffffffffu, (tail & 0x7FF) != 0)) {
+    low = INT_MAX;
+#pragma unroll
+    for (int i = 0; i < 4 * kGroups; ++i) {
+      const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v[i / 4][i % 4])) & ~(1ull << 63);
+      const int E = static_cast<int>(b >> 52), z = __ffsll(static_cast<long long>(b & ((1ull << 52) - 1)));
+      if (b != 0) low = min(low, max(E, 1) + (z != 0 ? z - 1 : 52));
+    }
+    low = __reduce_min_sync(0xffffffffu, low);
+  }
   if constexpr (kWarps > 1) {
-    if (lane == 0) smax[warp] = mb;
+    if (lane == 0) smax[warp] = mb, slow[warp] = low;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {
@@ -144,7 +168,15 @@ __global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restr
     finite = E != 0x7FF;
     e = E != 0 ? E - 1022 : -1022;
   }
-  if (wu == 0 && lane == 0) ex[r * ex_stride + c] = static_cast<int16_t>(finite ? e : kNonFinite);
+  if (wu == 0 && lane == 0) {
+    ex[r * ex_stride + c] = static_cast<int16_t>(finite ? e : kNonFinite);
+    if constexpr (kWarps > 1)
+      for (int w = 1; w < kWarps; ++w) low = min(low, slow[warp + w]);
+    int z = 0;
+    if (finite && mb != 0 && low != INT_MIN) z = min(max(low - 1075 + bits - e, 0) / 6, 7);
+    zeros[r * ex_stride + c] = static_cast<int8_t>(z);
+    if (z != 0) atomicMax(zmax, z);
+  }
   // the last chunk's last block is filled up with zeros
   const int64_t kw1 = (c == nch - 1) ? kb * kStepK : k1;
   // base of the chunk (of the whole operand unless it is triangular), its
@@ -238,18 +270,79 @@ __global__ void transpose_diag_blocks_kernel(const double* __restrict__ L, int64
 
 // -------------------------------------------------------------- product
 // Chinese remainder constants of the first `n` moduli: with y_m the inverse
-// of M / p_m modulo p_m, the integer x with residues r_m is M times the
-// fraction of sum_m r_m y_m / p_m.  limb[m] holds y_m / p_m to 72 binary
-// places: the first 32 (their products wrap modulo 1, as the fraction
-// does), then two limbs of 20, of which 15 products with a byte sum to less
-// than 2^31.  Cutting at 2^-72 leaves x off by about M 2^-65 = 2^44.6,
-// against roundings of the factors that add up to 2^51 over a full chunk.
+// of M / p_m modulo p_m, the integer x with residues r_m is sum_m r_m w_m, w_m =
+// y_m M / p_m, less a multiple of M, and x / M the fraction of sum_m r_m y_m / p_m.
+//
+// By the fraction: limb[m] holds y_m / p_m to 72 binary places: the first 32
+// (their products wrap modulo 1, as the fraction does), then two limbs of 20,
+// of which 15 products with a byte sum to less than 2^31.  Rounded at 2^-72 and
+// then at 2^-64 it leaves x off by at most 3.2 M 2^-64 (2^47.3 for 15 moduli),
+// to either side alike, against roundings of 48-bit factors that add up to 2^51
+// over a full chunk.
+//
+// Exactly: short factors are not rounded, and the fraction alone would lose
+// exact results that eight 6-bit digits had (1 * 1 and 3 * 5 came out as
+// 0.9999999999999988 and 14.999999999999995).  Pairs of at most nine digits
+// (kExactDigits) are put together in integers of 128 bits (combine_checked):
+// the fraction to 31 places (frac) gives the multiple of M and the bits of x
+// from 2^96 on, the sums modulo 2^96 the others.  Not every pair takes this
+// form because it costs 5 to 10 % where none is short (us: n = 3000, k = 200,
+// n0 = 256 514 by the fraction, 569 exactly; n = 16384, k = 256, n0 = 2048
+// 1215 and 1313; n = k = 8192 6280 and 6865).  An L of entries +-2^-14, all
+// pairs short: 690, 1596 and 7009 us.
 struct CrtConsts {
   int n;
   float p[kModuli], inv[kModuli];
   int limb[kModuli][3];
   double msc;  // M 2^-64
 };
+
+// Those of the exact form, which few products take: in constant memory, not
+// among the arguments of every launch.
+struct ExactConsts {
+  int frac[kModuli];        // y_m / p_m times 2^31
+  uint32_t w[kModuli][3];   // the words of w_m modulo 2^96, the lower two signed
+  uint32_t m[3];            // those of M
+  int top;                  // M 2^-79
+};
+
+constexpr int inverse_mod(int a, int p) {
+  int y = 1;
+  while (a * y % p != 1) ++y;  // a and p are coprime
+  return y;
+}
+
+// v modulo 2^96 = w[0] + w[1] 2^32 + w[2] 2^64 with the lower two read as
+// signed words.
+constexpr void low_words(unsigned __int128 v, uint32_t (&w)[3]) {
+  for (int i = 0; i < 3; ++i) {
+    w[i] = static_cast<uint32_t>(v);
+    v = (v >> 32) + (w[i] >> 31);  // a negative word takes one more of the next
+  }
+}
+
+constexpr unsigned __int128 modulus_product(int n) {
+  unsigned __int128 M = 1;
+  for (int m = 0; m < n; ++m) M *= static_cast<unsigned>(kP[m]);
+  return M;
+}
+
+constexpr ExactConsts make_exact_consts(int n) {
+  ExactConsts c{};
+  const unsigned __int128 M = modulus_product(n);
+  for (int m = 0; m < n; ++m) {
+    const unsigned p = static_cast<unsigned>(kP[m]);
+    const unsigned y = static_cast<unsigned>(inverse_mod(static_cast<int>((M / p) % p), kP[m]));
+    c.frac[m] = static_cast<int>(((static_cast<uint64_t>(y) << 32) / p + 1) >> 1);
+    low_words(M / p * y, c.w[m]);
+  }
+  low_words(M, c.m);
+  c.top = static_cast<int>(static_cast<int64_t>(M >> 79));
+  return c;
+}
+
+__constant__ ExactConsts kExact[3] = {make_exact_consts(13), make_exact_consts(14), make_exact_consts(15)};
+
 
 struct ProductArgs {
   int M, N, K, R, C;        // sizes, row tiles (of 128 or, for CTA pairs, 256 rows) and column tiles
@@ -270,6 +363,8 @@ struct ProductArgs {
   int64_t a_ex;
   const int16_t* eB;
   int64_t b_ex;
+  const int8_t *zA, *zB;    // zero digits of their factors, beside the exponents
+  const int *zmaxA, *zmaxB; // the most that a row of either operand has
   double* Y;
   int64_t ldy;
   const double* S;
@@ -282,9 +377,9 @@ struct ProductArgs {
 
 // Control words: the list position below which every item has been taken,
 // the output tiles finished (read together, 8 bytes), the CTAs that have
-// ended.
+// ended; kZeros: a zmax for B, which stays.
 constexpr long long kLingerNs = 20000;
-constexpr int kHead = 0, kReady = 1, kExited = 2, kCtrlWords = 64;
+constexpr int kHead = 0, kReady = 1, kExited = 2, kZeros = 4, kCtrlWords = 64;
 
 constexpr int kMaxRegs = 96;  // 19 warps: five on one scheduler, whose file holds 512 registers a lane
 
@@ -363,17 +458,135 @@ __device__ __forceinline__ int signed_byte(uint32_t w, int j) {
 // x 2^n where the result may leave the normal range.
 __device__ __noinline__ double scaled_slow(double x, double msc, int n) { return ldexp(x * msc, n); }
 
+// x 2^sc, rounded to the nearest double, from the sums over an output's
+// residues (S: with frac, A0 .. A2: with the words of w).  frac's roundings
+// leave x / M off by at most 2^-21.5, and |x| < 0.36 M: the nearest integer to
+// S is the multiple of M, and the error of x's bits from 2^64 on is below 2^25.
+__device__ __forceinline__ double exact_value(const ExactConsts& k, long long S, long long A0, long long A1, uint32_t A2,
+                                              int sc) {
+  const int q = static_cast<int>((S + (1ll << 30)) >> 31);
+  const long long frac = S - (static_cast<long long>(q) << 31);
+  A0 -= static_cast<long long>(q) * static_cast<int>(k.m[0]);
+  A1 -= static_cast<long long>(q) * static_cast<int>(k.m[1]);
+  A2 -= static_cast<uint32_t>(q) * k.m[2];
+  A1 += A0 >> 32;
+  A2 += static_cast<uint32_t>(A1 >> 32);
+  // x = hi 2^64 + lo, the bits of hi from 32 on from the fraction
+  const long long h = (frac * k.top) >> 16;
+  long long hi = h + static_cast<int>(A2 - static_cast<uint32_t>(h));
+  unsigned long long lo = (static_cast<unsigned long long>(A1) << 32) | static_cast<uint32_t>(A0);
+  const bool neg = hi < 0;
+  if (neg) {
+    lo = 0 - lo;
+    hi = ~hi + (lo == 0);
+  }
+  if (hi == 0 && lo == 0) return 0.0;
+  // the 64 bits from the leading one on; hi is below 2^44
+  const int lz = hi != 0 ? __clzll(hi) : __clzll(static_cast<long long>(lo));
+  const unsigned long long t = hi != 0 ? (static_cast<unsigned long long>(hi) << lz) | (lo >> (64 - lz)) : lo << lz;
+  const bool rest = (t & 0x3FF) != 0 || (hi != 0 && (lo << lz) != 0);
+  const long long m = static_cast<long long>((t >> 11) + ((t >> 10) & 1 & (rest ? 1 : t >> 11)));
+  const int e = (hi != 0 ? 127 : 63) - lz;  // x = 1.f 2^e
+  const int E = e + sc >= -1022 && e + sc <= 1022 ? e + sc : e;
+  const double v = __longlong_as_double(m + (static_cast<long long>(E + 1022) << 52));
+  return E == e + sc ? (neg ? -v : v) : scaled_slow(neg ? -v : v, 1.0, sc);
+}
+
+// The sums of an output's residues with the limbs.
+struct Fraction {
+  uint32_t s0 = 0;
+  int s1 = 0, s2 = 0;
+  __device__ __forceinline__ void add(const CrtConsts& k, int m, int r) {
+    s0 += static_cast<uint32_t>(r) * static_cast<uint32_t>(k.limb[m][0]);
+    s1 += r * k.limb[m][1];
+    s2 += r * k.limb[m][2];
+  }
+  // the fraction to 64 binary places, as a signed number in [-1/2, 1/2)
+  __device__ __forceinline__ double value() const {
+    return static_cast<double>(static_cast<long long>(
+        (static_cast<unsigned long long>(s0) << 32) + (static_cast<unsigned long long>(static_cast<long long>(s1)) << 12) +
+        static_cast<unsigned long long>(static_cast<long long>((s2 + 128) >> 8))));
+  }
+};
+
+// One output from its base (S, or S - dg X) and its product's fraction f; ea
+// and eb are the exponents of its factors.
+__device__ __forceinline__ double apply_fraction(const ProductArgs& a, double f, int ea, int eb, double dg, double base) {
+  const long long sign = a.mode == kRnsDiag ? 0 : static_cast<long long>(1ull << 63);
+  const int sc = ea + eb - a.bits;
+  if (sc >= -1050 && sc <= 970) {
+    // msc = 1.x 2^31 to 1.x 2^45: the scale is normal in this range
+    const double scale = __longlong_as_double((__double_as_longlong(a.k.msc) + (static_cast<long long>(sc) << 52)) ^ sign);
+    // the diagonal term, usually the larger, is not rounded on its own
+    return a.mode == kRnsDiag ? fma(dg, base, f * scale) : fma(f, scale, base);
+  }
+  if (ea == kNonFinite || eb == kNonFinite) return __longlong_as_double(0x7FF8000000000000ll);
+  const double v = scaled_slow(f, a.k.msc, sc);
+  return a.mode == kRnsDiag ? fma(dg, base, v) : base - v;
+}
+
+// combine_tile where the operands' zero digits allow exact pairs: a pair's
+// product exactly if its factors are short, the others' by the fraction, so
+// that an output depends on its own row and column alone.  A role of its own:
+// a call from combine_tile's loop, never taken, made the kernel spill and cost
+// 2 % at n = 3000, k = 200.
+template <int BN>
+__device__ __forceinline__ void combine_checked(const ProductArgs& a, int tile, int tm, int tn, int row, int cg0, int cg1) {
+  const int grow = tm * 128 + row;
+  if (grow >= a.M) return;
+  const ExactConsts& k = kExact[a.k.n - 13];
+  const int ea = a.eA[static_cast<int64_t>(grow) * a.a_ex], za = a.zA[static_cast<int64_t>(grow) * a.a_ex];
+  const double dg = a.mode != kRnsUpdate ? a.dg[grow] : 0.0;
+#pragma unroll 1
+  for (int cg = cg0; cg < cg1; ++cg) {
+    const int col0 = tn * BN + cg * 8;
+    const uint2* rp = a.resid + (static_cast<int64_t>(tile) * a.k.n * (BN / 8) + cg) * 128 + row;
+    uint2 rv[kModuli];
+#pragma unroll
+    for (int m = 0; m < kModuli; ++m)
+      rv[m] = m < a.k.n ? __ldcg(rp + static_cast<int64_t>(m) * (BN / 8) * 128) : make_uint2(0, 0);
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+      const int64_t col = col0 + j;
+      if (col >= a.N) break;
+      const int eb = a.eB[col * a.b_ex];
+      double base = a.S[col * a.lds + grow];
+      if (a.mode == kRnsResidual) base = fma(-dg, a.X[col * a.ldx + grow], base);
+      double y;
+      if (za + a.zB[col * a.b_ex] >= kExactDigits) {  // both finite
+        long long S = 0, A0 = 0, A1 = 0;
+        uint32_t A2 = 0;
+#pragma unroll
+        for (int m = 0; m < kModuli; ++m) {
+          const int r = signed_byte(j < 4 ? rv[m].x : rv[m].y, j & 3);
+          S += static_cast<long long>(r) * k.frac[m];
+          A0 += static_cast<long long>(r) * static_cast<int>(k.w[m][0]);
+          A1 += static_cast<long long>(r) * static_cast<int>(k.w[m][1]);
+          A2 += static_cast<uint32_t>(r) * k.w[m][2];
+        }
+        const double v = exact_value(k, S, A0, A1, A2, ea + eb - a.bits);
+        y = a.mode == kRnsDiag ? fma(dg, base, v) : base - v;
+      } else {
+        Fraction f;
+#pragma unroll
+        for (int m = 0; m < kModuli; ++m) f.add(a.k, m, signed_byte(j < 4 ? rv[m].x : rv[m].y, j & 3));
+        y = apply_fraction(a, f.value(), ea, eb, dg, base);
+      }
+      a.Y[col * a.ldy + grow] = y;
+    }
+  }
+}
+
 // Puts the integer products of the 8-column groups [cg0, cg1) of an output
-// tile together from their residues and applies them, a row per lane.  Per output: 15 byte extractions and 45 multiply-adds,
-// then a conversion and one or two FP64 operations.
+// tile together from their residues and applies them, a row per lane.  Per
+// output: 15 byte extractions and 45 multiply-adds, then a conversion and one
+// or two FP64 operations.
 template <int BN>
 __device__ __forceinline__ void combine_tile(const ProductArgs& a, int tile, int tm, int tn, int row, int cg0, int cg1) {
   const int grow = tm * 128 + row;
   if (grow >= a.M) return;
   const int ea = a.eA[static_cast<int64_t>(grow) * a.a_ex];
   const double dg = a.mode != kRnsUpdate ? a.dg[grow] : 0.0;
-  const long long msc = __double_as_longlong(a.k.msc);
-  const long long sign = a.mode == kRnsDiag ? 0 : static_cast<long long>(1ull << 63);
   const int nm = a.k.n;
 #pragma unroll 1
   for (int cg = cg0; cg < cg1; ++cg) {
@@ -403,36 +616,11 @@ __device__ __forceinline__ void combine_tile(const ProductArgs& a, int tile, int
     double* Yp = a.Y + static_cast<int64_t>(col0) * a.ldy + grow;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      uint32_t s0 = 0;
-      int s1 = 0, s2 = 0;
+      Fraction f;
 #pragma unroll
-      for (int m = 0; m < kModuli; ++m) {
-        const int r = signed_byte(j < 4 ? rv[m].x : rv[m].y, j & 3);
-        s0 += static_cast<uint32_t>(r * a.k.limb[m][0]);
-        s1 += r * a.k.limb[m][1];
-        s2 += r * a.k.limb[m][2];
-      }
+      for (int m = 0; m < kModuli; ++m) f.add(a.k, m, signed_byte(j < 4 ? rv[m].x : rv[m].y, j & 3));
       if (j >= ncol) continue;
-      // the fraction to 64 binary places, as a signed number in [-1/2, 1/2)
-      const long long F = static_cast<long long>((static_cast<unsigned long long>(s0) << 32) +
-                                                 (static_cast<unsigned long long>(static_cast<long long>(s1)) << 12) +
-                                                 static_cast<unsigned long long>(static_cast<long long>(s2 >> 8)));
-      const int eb = eb8[j];
-      const int sc = ea + eb - a.bits;
-      const double f = static_cast<double>(F);
-      double y;
-      if (sc >= -1050 && sc <= 970) {
-        // msc = 1.x 2^31 to 1.x 2^45: the scale is normal in this range
-        const double scale = __longlong_as_double((msc + (static_cast<long long>(sc) << 52)) ^ sign);
-        // the diagonal term, usually the larger, is not rounded on its own
-        y = a.mode == kRnsDiag ? fma(dg, base[j], f * scale) : fma(f, scale, base[j]);
-      } else if (ea == kNonFinite || eb == kNonFinite) {
-        y = __longlong_as_double(0x7FF8000000000000ll);
-      } else {
-        const double v = scaled_slow(f, a.k.msc, sc);
-        y = a.mode == kRnsDiag ? fma(dg, base[j], v) : base[j] - v;
-      }
-      Yp[static_cast<int64_t>(j) * a.ldy] = y;
+      Yp[static_cast<int64_t>(j) * a.ldy] = apply_fraction(a, f.value(), ea, eb8[j], dg, base[j]);
     }
   }
 }
@@ -662,17 +850,25 @@ __global__ void __maxnreg__(kMaxRegs)
   } else if (warp < 2 + S::kEpiWarps + S::kCombWarps) {
     const int w = warp - 2 - S::kEpiWarps;
     const int groups = a.item_cols / 16;  // 8-column groups per warp
-    for (int i = 0;; ++i) {
-      const int q = i & 1;
-      if (!tc::mbar_wait(&qfull_bar[q], (i >> 1) & 1, abort_flag)) break;
-      const int item = queue[q];
-      if (item < 0) break;
-      const int tile = item / items;
-      const int cg0 = item % items * (2 * groups) + (w >> 2) * groups;
-      combine_tile<BN>(a, tile, tile / a.C, tile % a.C, (w & 3) * 32 + lane, cg0, cg0 + groups);
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&qempty_bar[q]);
-    }
+    // zero digits are rare: the operands' most settle which form runs
+    auto combine_items = [&](auto checked) {
+      for (int i = 0;; ++i) {
+        const int q = i & 1;
+        if (!tc::mbar_wait(&qfull_bar[q], (i >> 1) & 1, abort_flag)) break;
+        const int item = queue[q];
+        if (item < 0) break;
+        const int tile = item / items;
+        const int cg0 = item % items * (2 * groups) + (w >> 2) * groups;
+        if constexpr (decltype(checked)::value)
+          combine_checked<BN>(a, tile, tile / a.C, tile % a.C, (w & 3) * 32 + lane, cg0, cg0 + groups);
+        else
+          combine_tile<BN>(a, tile, tile / a.C, tile % a.C, (w & 3) * 32 + lane, cg0, cg0 + groups);
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&qempty_bar[q]);
+      }
+    };
+    if (*a.zmaxA + *a.zmaxB >= kExactDigits) combine_items(std::true_type());
+    else combine_items(std::false_type());
   } else {
     int pushed = 0;
     // true once the item `back` before the next one has been combined
@@ -788,21 +984,19 @@ rns::ResidueConsts make_residue_consts() {
 rns::CrtConsts make_crt_consts(int n) {
   rns::CrtConsts c{};
   c.n = n;
-  unsigned __int128 M = 1;
-  for (int m = 0; m < n; ++m) M *= static_cast<unsigned>(kP[m]);
+  const unsigned __int128 M = rns::modulus_product(n);
   for (int m = 0; m < n; ++m) {
     const int p = kP[m];
     c.p[m] = static_cast<float>(p);
     c.inv[m] = 1.f / static_cast<float>(p);
-    const int g = static_cast<int>((M / static_cast<unsigned>(p)) % static_cast<unsigned>(p));
-    int y = 1;
-    while (g * y % p != 1) ++y;  // p and M / p are coprime
-    uint64_t rem = static_cast<uint64_t>(y);
+    uint64_t rem = static_cast<uint64_t>(
+        rns::inverse_mod(static_cast<int>((M / static_cast<unsigned>(p)) % static_cast<unsigned>(p)), p));
     for (int q = 0; q < 3; ++q) {
       rem <<= q == 0 ? 32 : 20;
       c.limb[m][q] = static_cast<int>(static_cast<uint32_t>(rem / static_cast<unsigned>(p)));
       rem %= static_cast<unsigned>(p);
     }
+    c.limb[m][2] += 2 * rem >= static_cast<unsigned>(p);  // to nearest
   }
   c.msc = static_cast<double>(M) * 0x1p-64;
   return c;
@@ -856,7 +1050,7 @@ cudaError_t launch_residues(const double* src, int64_t ld, int64_t K, const RnsO
                             const rns::ResidueConsts& rc, cudaStream_t s) {
   const int64_t units = o.rows * o.nch, per = 8 / kWarps;
   return launch_dependent(rns::residue_rows_kernel<kWarps>, dim3(static_cast<unsigned>((units + per - 1) / per)), dim3(256),
-                          0, s, 1, src, ld, o.rows, K, o.nch, o.kc, o.ex_ld, o.res, o.kb, o.ex, c.moduli, c.bits,
+                          0, s, 1, src, ld, o.rows, K, o.nch, o.kc, o.ex_ld, o.res, o.kb, o.ex, o.zeros, o.zmax, c.moduli, c.bits,
                           o.tri ? 1 : 0, vec ? 1 : 0, rc);
 }
 
@@ -876,7 +1070,9 @@ static size_t residue_bytes(int64_t rows, int64_t K, int64_t kc, bool tri) {
 }
 
 size_t rns_operand_bytes(int64_t rows, int64_t K, int64_t kc, bool tri) {
-  return residue_bytes(rows, K, kc, tri) + al256(sizeof(int16_t) * static_cast<size_t>(rows) * ((K + kc - 1) / kc));
+  // residues, a word for zmax, exponents, zero digits
+  const size_t pairs = static_cast<size_t>(rows) * ((K + kc - 1) / kc);
+  return residue_bytes(rows, K, kc, tri) + 256 + al256(sizeof(int16_t) * pairs) + al256(pairs);
 }
 
 RnsOperand rns_operand_view(void* base, int64_t rows, int64_t K, int64_t kc, bool tri) {
@@ -888,7 +1084,10 @@ RnsOperand rns_operand_view(void* base, int64_t rows, int64_t K, int64_t kc, boo
   o.nch = o.ex_ld = (K + kc - 1) / kc;
   o.tri = tri;
   o.res = static_cast<__nv_bfloat16*>(base);
-  o.ex = reinterpret_cast<int16_t*>(static_cast<unsigned char*>(base) + residue_bytes(rows, K, kc, tri));
+  unsigned char* p = static_cast<unsigned char*>(base) + residue_bytes(rows, K, kc, tri);
+  o.zmax = reinterpret_cast<int*>(p);
+  o.ex = reinterpret_cast<int16_t*>(p + 256);
+  o.zeros = reinterpret_cast<int8_t*>(p + 256 + al256(sizeof(int16_t) * static_cast<size_t>(rows) * o.nch));
   return o;
 }
 
@@ -902,6 +1101,7 @@ RnsOperand rns_chunk(const RnsOperand& o, int64_t c) {
   v.nch = 1;
   v.res += kModuli * o.kc * (c * o.rows - o.kc * (c * (c - 1) / 2));
   v.ex += k0 * o.ex_ld + c;
+  v.zeros += k0 * o.ex_ld + c;
   return v;
 }
 
@@ -930,7 +1130,8 @@ static cudaError_t transpose_and_reduce(const double* L, int64_t ldl, int64_t n,
   dim3 grid(static_cast<unsigned>((n + 31) / 32), static_cast<unsigned>((n + 31) / 32));
   rns::transpose_lower_kernel<<<grid, dim3(32, 8), 0, s>>>(L, ldl, tmp, n, n0, o.kc);
   count_launch();
-  const cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemsetAsync(o.zmax, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   return rns_rows(tmp, n, n, o, RnsClass{kModuli, kBitsFull}, s);
 }
@@ -951,7 +1152,8 @@ cudaError_t rns_inverse_block_rows(const double* Lt, int64_t ldt, int64_t n, int
   dim3 grid(static_cast<unsigned>((n0 + 31) / 32), static_cast<unsigned>((n + 31) / 32));
   rns::transpose_diag_blocks_kernel<<<grid, dim3(32, 8), 0, s>>>(Lt, ldt, tmp, diag, n, n0);
   count_launch();
-  const cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemsetAsync(inv.zmax, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   return rns_rows(tmp, n0, n0, inv, RnsClass{kModuli, kBitsFull}, s);
 }
@@ -970,6 +1172,7 @@ RnsScratch rns_scratch_view(void* base, int64_t M, int64_t N) {
   RnsScratch sc;
   sc.tiles = tile_plan(M, N).cap;
   sc.ctrl = static_cast<int*>(base);
+  sc.zmax = sc.ctrl + rns::kZeros;
   sc.resid = static_cast<unsigned char*>(base) + control_bytes(sc.tiles);
   return sc;
 }
@@ -1019,6 +1222,9 @@ cudaError_t rns_product(const RnsProduct& p, const RnsScratch& sc, int* err, cud
   a.eA = p.A.ex + p.a_row0 * p.A.ex_ld + p.a_k0 / p.A.kc;
   a.a_ex = p.A.ex_ld;
   a.b_ex = p.B.ex_ld;
+  a.zA = p.A.zeros + p.a_row0 * p.A.ex_ld + p.a_k0 / p.A.kc;
+  a.zmaxA = p.A.zmax;
+  a.zmaxB = p.B.zmax;
   a.ldy = p.ldy;
   a.lds = p.lds;
   a.dg = p.dg;
@@ -1032,7 +1238,9 @@ cudaError_t rns_product(const RnsProduct& p, const RnsScratch& sc, int* err, cud
     a.GC = std::min(a.C, 8);
     a.GR = std::max(1, (pair ? 32 : 64) / a.GC);
     a.b_row0 = static_cast<int>(p.b_row0 + col0);
-    a.eB = p.B.ex + (p.b_row0 + col0) * p.B.ex_ld + p.b_k0 / p.B.kc;
+    const int64_t b_at = (p.b_row0 + col0) * p.B.ex_ld + p.b_k0 / p.B.kc;
+    a.eB = p.B.ex + b_at;
+    a.zB = p.B.zeros + b_at;
     a.Y = p.Y + col0 * p.ldy;
     a.S = p.S + col0 * p.lds;
     a.X = p.X ? p.X + col0 * p.ldx : nullptr;
@@ -1112,9 +1320,10 @@ extern "C" int trsm_residual_sliced(const double* L_dev, int64_t n, int64_t ldl,
   cudaError_t e = trsm::ws_alloc(reinterpret_cast<void**>(&buf), lb + xb + tb + db + sb, s);
   if (e != cudaSuccess) return -3;
   const trsm::RnsOperand Ls = trsm::rns_operand_view(buf, n, n, trsm::kChunk, true);
-  const trsm::RnsOperand Xs = trsm::rns_operand_view(buf + lb, k, n);
+  trsm::RnsOperand Xs = trsm::rns_operand_view(buf + lb, k, n);
   double* diag = reinterpret_cast<double*>(buf + lb + xb + tb);
   const trsm::RnsScratch sc = trsm::rns_scratch_view(buf + lb + xb + tb + db, n, k);
+  Xs.zmax = sc.zmax;
   e = trsm::rns_scratch_clear(sc, s);
   if (e == cudaSuccess) e = trsm::rns_lower_rows(L_dev, ldl, n, Ls, reinterpret_cast<double*>(buf + lb + xb), s);
   if (e == cudaSuccess) {

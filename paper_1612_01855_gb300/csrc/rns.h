@@ -16,9 +16,13 @@
 //   * reduced modulo p again, the sums are the residues of the integer
 //     product, whose absolute value is at most 2^(11 + bitsA + bitsB), below
 //     half the product M of the moduli: the Chinese remainder theorem gives
-//     it back exactly, and it is scaled and applied in FP64.
-// The only errors are the roundings of the factors to `bits` bits and the
-// final FP64 operations.
+//     it back, and it is scaled and applied in FP64.
+// The errors are the roundings of the factors to `bits` bits, the integer
+// product's to 3.2 M 2^-64 at most (about 2^-49 of the product of the two
+// maxima, to either side alike) and the final FP64 operations.  Short factors,
+// nine 6-bit digits a pair from their maxima down (24 and 30 bits, say, or
+// integers below 2^24 both), are not rounded and give the double next to their
+// product: integer and dyadic systems keep their exact results.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -46,6 +50,8 @@ constexpr int kBitsFull = 48;  // integer bits of the plan's operands and of an 
 struct RnsOperand {
   __nv_bfloat16* res = nullptr;  // [kModuli][kb][rows][64]
   int16_t* ex = nullptr;         // exponent of (row, chunk) at ex[row ex_ld + chunk]
+  int8_t* zeros = nullptr;       // in the same places: 6-bit digits (0 to 7) that end all its integers in zeros
+  int* zmax = nullptr;           // at least the largest of them; zero before the first residues are made
   int64_t rows = 0, K = 0, kb = 0, nch = 0, kc = kChunk, ex_ld = 0;  // kb: blocks of 64 along K
   bool tri = false;
 };
@@ -120,10 +126,12 @@ struct RnsProduct {
 
 // Scratch of the products of at most M rows and exactly N columns: control
 // words and the residues of the sums.  The control words must be zero before
-// the first product (rns_scratch_clear); every product leaves them zero.
+// the first product (rns_scratch_clear); every product leaves them zero (zmax
+// as it is).
 // Products that may overlap need scratch of their own.
 struct RnsScratch {
   int* ctrl = nullptr;
+  int* zmax = nullptr;  // a word for the zmax of an operand made again and again; rns_scratch_clear zeroes it
   void* resid = nullptr;
   int64_t tiles = 0;  // output tiles it holds
 };

@@ -160,8 +160,9 @@ int solve_sliced(trsm_plan_s* h, const double* B, int64_t k, int64_t ldb, double
   for (int64_t j0 = 0; j0 < k && e == cudaSuccess; j0 += kp) {
     const Panel pn{B + j0 * ldb, ldb, X + j0 * ldx, ldx, std::min(kp, k - j0)};
     // the residues of W(S_i) are dead once X(S_i) is there: one buffer
-    const RnsOperand P = rns_operand_view(ws + wbytes, pn.k, nb, nb);
+    RnsOperand P = rns_operand_view(ws + wbytes, pn.k, nb, nb);
     const RnsScratch sc = rns_scratch_view(scratch, n, pn.k);
+    P.zmax = sc.zmax;
     e = rns_scratch_clear(sc, s);
     if (e == cudaSuccess) e = solve_panel(h, pn, W, ld, P, sc, err, s);
   }
