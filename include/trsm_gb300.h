@@ -57,8 +57,8 @@ extern "C" {
 /* Residual of the mixed-precision solve. */
 /* The sliced residuals run on the bf16 tensor cores in integer arithmetic: L
  * to 48 bits of each (row, 2048-wide chunk) maximum, X to 42 bits of each
- * (column, chunk) maximum in the seven-plane class, 48 in the eight-plane
- * class (35 in the classes of five and six), products to 2^-49 of the
+ * (column, chunk) maximum in the six- and seven-plane classes, 48 in the
+ * eight-plane class (35 in the five-plane class), products to 2^-49 of the
  * maxima's, exactly for factors of up to nine 6-bit digits a pair. */
 #define TRSM_RESIDUAL_SLICED 0   /* FP64-class: the seven-plane class */
 #define TRSM_RESIDUAL_FP64 1     /* FP64 fused multiply-add                                */
@@ -66,10 +66,11 @@ extern "C" {
 #define TRSM_RESIDUAL_ADAPTIVE 3 /* SLICED until the updates stagnate above tol or their contraction
                                     stalls (an update ten times above the last contraction's
                                     prediction), then SLICED8 */
-/* As ADAPTIVE, but an early residual takes the class of 5 or 6 planes (13
- * tensor-core products instead of 14; about 2^-38 of |B| + |L||X|) while the iterate's error, estimated from the last update and its
- * contraction, is far above what they resolve; 7 planes after that, 8 once
- * the updates stagnate. */
+/* As ADAPTIVE, but an early residual takes the class of 5 planes (13
+ * tensor-core products instead of 14; about 2^-38 of |B| + |L||X|) while the
+ * iterate's error, estimated from the last update and its contraction, is far
+ * above what it resolves (that of 6, with 7's products, nearer to it); 7
+ * planes after that, 8 once the updates stagnate. */
 #define TRSM_RESIDUAL_PROGRESSIVE 4
 /* Flag or-ed into `residual`: apply the FP64 inverses of the diagonal blocks
  * in FP32 arithmetic inside the inner solve (default: FP64 arithmetic). */

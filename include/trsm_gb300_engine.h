@@ -32,14 +32,14 @@ int trsm_tc_gemm_selftest(int mode, const void* A_dev, const void* B_dev, float*
 
 /* FP64-class residual R = B - tril(L) X on the BF16 tensor cores: the
  * strictly lower L and X are rounded to integers of 48 bits and, for planes
- * = 5 .. 8, of 35, 35, 42 or 48 bits per (row, 2048-wide chunk of K) with a
- * power-of-two exponent each; their residues modulo 13, 13, 14 or 15 moduli
+ * = 5 .. 8, of 35, 42, 42 or 48 bits per (row, 2048-wide chunk of K) with a
+ * power-of-two exponent each; their residues modulo 13, 14, 14 or 15 moduli
  * are multiplied with exact FP32 sums, and the chunk's integer product is put
  * together from them (to 3.2 2^-64 of the moduli's product, exactly for
  * factors of up to nine 6-bit digits a pair) and applied in FP64 (after Ozaki, Uchino &
  * Imamura 2025); the diagonal of L is applied in FP64.  Relative error about
- * 2^-45 (7 planes) or 2^-50 (8 planes) of (|B| + |L| |X|), about 2^-38 with
- * 5 or 6.
+ * 2^-45 (6 or 7 planes) or 2^-50 (8 planes) of (|B| + |L| |X|), about 2^-38
+ * with 5.
  *   L_dev n x n column-major (lower triangle read), X_dev, B_dev, R_dev
  *   n x k column-major.  Allocates its residue buffers stream-ordered.
  *   Asynchronous; err_dev as for the self-test; -1 for bad arguments. */

@@ -64,12 +64,12 @@ RnsOperand rns_chunk(const RnsOperand& o, int64_t c);
 // product of the accuracy class of P 6-bit digits takes (P = 5 .. 8; the
 // left factor, the plan's, always has kBitsFull bits).  M / 2 has to exceed
 // 2^(11 + 48 + bits): 13, 14 and 15 moduli make 2^83.5, 2^90.6 and 2^97.6 of
-// 2^(bitsA + bitsB).
+// 2^(bitsA + bitsB): six digits are one bit too many for 13 moduli.
 struct RnsClass {
   int moduli, bits;
 };
 inline RnsClass rns_class(int planes) {
-  return planes <= 6 ? RnsClass{13, 35} : planes == 7 ? RnsClass{14, 42} : RnsClass{15, kBitsFull};
+  return planes <= 5 ? RnsClass{13, 35} : planes <= 7 ? RnsClass{14, 42} : RnsClass{15, kBitsFull};
 }
 
 // Residues of `rows` rows of FP64 values (row r contiguous from src + r ld)
@@ -143,7 +143,7 @@ cudaError_t rns_product(const RnsProduct& p, const RnsScratch& sc, int* err, cud
 // R = B - L X with the strictly lower part of L given by its residue rows
 // (Ls: n x n), its diagonal as a vector, and X by its residue rows (Xs: k
 // rows of length n, made in the class of `planes`) and by itself; R, B, X
-// column-major n x k.  `planes` (5 to 8) sets the accuracy: X to 35, 35, 42
+// column-major n x k.  `planes` (5 to 8) sets the accuracy: X to 35, 42, 42
 // or 48 bits of each (column, chunk) maximum.
 cudaError_t rns_residual(const RnsOperand& Ls, const double* diag, const RnsOperand& Xs, const double* X, int64_t ldx,
                          const double* B, int64_t ldb, double* R, int64_t ldr, int planes, const RnsScratch& sc,

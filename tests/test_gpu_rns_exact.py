@@ -109,3 +109,15 @@ def test_cancellation_and_range(cuda_lib, planes):
     want[n - 1] = B[n - 1]
     R = _residual(cuda_lib, L, X, B, planes)
     assert np.array_equal(R, want)
+
+
+def test_six_plane_class_keeps_36_bits(cuda_lib):
+    """Six digits are 36 bits: columns of 36-bit integers under an L of +-1
+    (seven digits a pair) come out exactly."""
+    rng = np.random.default_rng(6)
+    n, k = 70, 9
+    L = np.tril(rng.choice([-1, 1], size=(n, n)))
+    X = rng.integers(-2 ** 36 + 1, 2 ** 36, size=(n, k)) | 1
+    B = rng.integers(-2 ** 40, 2 ** 40, size=(n, k))
+    R = _residual(cuda_lib, L, X, B, 6)
+    assert np.array_equal(R, (B - L @ X).astype(np.float64))
