@@ -126,6 +126,10 @@ cudaError_t ws_alloc(T** p, size_t bytes, cudaStream_t s) {
 // early, 1218 with the element-wise ones alone; refined n = 3000, k = 128:
 // 1295, 965, 925), and a CTA that waits must not hold tensor memory that one
 // of them still has to get.
+// Such a kernel runs beside the ones before it, so nothing they write is
+// read-only for its lifetime: it reads by plain loads, after its wait. No
+// __ldg and no const __restrict__ pointer (either allows the read-only path,
+// which need not see those writes, and a load that moves above the wait).
 // cluster: CTAs per cluster (1: none).
 template <class... KArgs, class... Args>
 cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -216,8 +216,8 @@ __device__ __forceinline__ double scale_pow2(double x, int n) {
 // with v rounded once to FP32 first: v - hi is then exact in FP32 and
 // hi + lo keeps 22 bits of v.  Rows on threadIdx.x (coalesced in D and in
 // Dt), columns on blockIdx.y.
-__global__ void pack_dt_f16_kernel(const double* __restrict__ D, int64_t ldd, int64_t s0, int m, int64_t k,
-                                   int64_t n0p, const unsigned long long* __restrict__ dmax, const int* panel_exp,
+__global__ void pack_dt_f16_kernel(const double* D, int64_t ldd, int64_t s0, int m, int64_t k,
+                                   int64_t n0p, const unsigned long long* dmax, const int* panel_exp,
                                    __half* __restrict__ Dt, float* __restrict__ gscale) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -297,7 +297,7 @@ __global__ void pack_inv_tf32_kernel(const double* __restrict__ Lt, int64_t ldt,
 // mid = tf32(w - hi), lo = w - hi - mid (every difference exact in FP32, and
 // the three planes hold all 24 bits of w).  Rows on threadIdx.x.
 template <int P>
-__global__ void pack_w_tf32_kernel(const float* __restrict__ W, int64_t ldw, int64_t s0, int m, int64_t k,
+__global__ void pack_w_tf32_kernel(const float* W, int64_t ldw, int64_t s0, int m, int64_t k,
                                    int64_t n0p, float* __restrict__ Wt) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -318,7 +318,7 @@ __global__ void pack_w_tf32_kernel(const float* __restrict__ W, int64_t ldw, int
 // The same with four rows per thread in 16-byte accesses (ldw, s0 and n0p
 // multiples of 4, W 16-byte aligned) and two columns in flight.
 template <int P>
-__global__ void pack_w_tf32_vec_kernel(const float* __restrict__ W, int64_t ldw, int64_t s0, int m, int64_t k,
+__global__ void pack_w_tf32_vec_kernel(const float* W, int64_t ldw, int64_t s0, int m, int64_t k,
                                        int64_t n0p, float* __restrict__ Wt) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -355,7 +355,7 @@ __global__ void pack_w_tf32_vec_kernel(const float* __restrict__ W, int64_t ldw,
 // split bf16; split fp16 takes pack_dt_f16_kernel): the tensor-core
 // diagonal multiply writes D alone.
 template <int kMode>
-__global__ void pack_dt_kernel(const double* __restrict__ D, int64_t ldd, int64_t s0, int m, int64_t k, int64_t n0p,
+__global__ void pack_dt_kernel(const double* D, int64_t ldd, int64_t s0, int m, int64_t k, int64_t n0p,
                                typename LowP<kMode>::T* __restrict__ Dt) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -393,7 +393,7 @@ __global__ void extract_diag_kernel(const double* __restrict__ L, int64_t ldl, i
 // every leading dimension is even and every base 16-byte aligned (kVec);
 // the columns are spread over grid.y, several per CTA (grid_pairs).
 template <bool kVec>
-__global__ void to_float_kernel(const double* __restrict__ R, int64_t ldr, float* __restrict__ W,
+__global__ void to_float_kernel(const double* R, int64_t ldr, float* __restrict__ W,
                                 int64_t ldw, int64_t n, int64_t k) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -707,7 +707,7 @@ void launch_s_step(bool s32, const double* Lt, int64_t ldt, const float* Lf, int
 // maximum; it is stored as ~0).  Integer maxima keep the FP64 pipe for the
 // additions alone.
 template <bool kVec, bool kFirst>
-__global__ void correct_kernel(double* __restrict__ X, int64_t ldx, const double* __restrict__ D,
+__global__ void correct_kernel(double* __restrict__ X, int64_t ldx, const double* D,
                                int64_t ldd, int64_t n, int64_t k,
                                unsigned long long* __restrict__ norms) {
   grid_launch_dependents();

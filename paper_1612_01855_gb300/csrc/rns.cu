@@ -90,7 +90,7 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
 // *zmax.  A value with one of its lowest 11 bits set leaves none, which settles
 // nearly every warp with one vote.
 template <int kWarps>
-__global__ void __launch_bounds__(256) residue_rows_kernel(const double* __restrict__ src, int64_t ld, int64_t rows,
+__global__ void __launch_bounds__(256) residue_rows_kernel(const double* src, int64_t ld, int64_t rows,
                                                            int64_t K, int64_t nch, int64_t kc, int64_t ex_stride,
                                                            __nv_bfloat16* __restrict__ dst, int64_t kb,
                                                            int16_t* __restrict__ ex, int8_t* __restrict__ zeros,
@@ -602,7 +602,7 @@ __device__ __forceinline__ void combine_tile(const ProductArgs& a, int tile, int
     const int16_t* eBp = a.eB + static_cast<int64_t>(col0) * a.b_ex;
     int eb8[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) eb8[j] = j < ncol ? __ldg(eBp + static_cast<int64_t>(j) * a.b_ex) : 0;
+    for (int j = 0; j < 8; ++j) eb8[j] = j < ncol ? eBp[static_cast<int64_t>(j) * a.b_ex] : 0;
     const double* Sp = a.S + static_cast<int64_t>(col0) * a.lds + grow;
     double base[8];
 #pragma unroll

@@ -94,7 +94,7 @@ struct StoreF32Epi {
     if (r >= M) return;
     float* base = C + static_cast<int64_t>(tn * BN + sl * 16) * ldc + r;
     const int ncol = min(16, N - (tn * BN + sl * 16));
-    const float a = scale ? alpha * __ldg(scale) : alpha;
+    const float a = scale ? alpha * *scale : alpha;
     // all loads of the slab first, so that their latencies overlap
     float old[16];
 #pragma unroll
