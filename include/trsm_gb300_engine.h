@@ -58,6 +58,17 @@ int trsm_residual_sliced(const double* L_dev, int64_t n, int64_t ldl, const doub
 int trsm_residual_plan(trsm_handle_t h, const double* X_dev, int64_t k, int64_t ldx, const double* B_dev,
                        int64_t ldb, double* R_dev, int64_t ldr, int planes, int* err_dev, void* stream);
 
+/* The two forms of trsm_solve, for comparison (no counterpart in the paper):
+ * trsm_solve_form runs the tile tasks with S = CW = 0, else the solve by
+ * columns with S CTAs (1 .. 8, at most the plan's block rows) on every CW
+ * columns (1 .. 8); TRSM_EINVAL where that form cannot run (n0 above 256,
+ * several blocks of odd order, or rows that do not fit in shared memory).
+ * Both give the bits of trsm_solve.  trsm_solve_form_choice: the S and CW that
+ * trsm_solve takes for k columns, 0 and 0 for the tile tasks. */
+int trsm_solve_form(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, double* X_dev, int64_t ldx, int S,
+                    int CW, void* stream);
+int trsm_solve_form_choice(trsm_handle_t h, int64_t k, int* S, int* CW);
+
 /* Failure-detection self-test (no counterpart in the paper): launches one
  * small kernel whose wait can never be satisfied, with a time limit of
  * limit_us microseconds (1 .. 2e6), and reports what the library would:

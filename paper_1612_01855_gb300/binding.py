@@ -91,6 +91,8 @@ SIGNATURES = {
     "trsm_fp64_peak": (_int, [_int, ctypes.POINTER(ctypes.c_double), _vp]),
     "trsm_fp32_peak": (_int, [_int, ctypes.POINTER(ctypes.c_double), _vp]),
     "trsm_tc_gemm_selftest": (_int, [_int, _vp, _vp, _vp, _i64, _i64, _i64, _vp, _vp]),
+    "trsm_solve_form": (_int, [_vp, _dp, _i64, _i64, _dp, _i64, _int, _int, _vp]),
+    "trsm_solve_form_choice": (_int, [_vp, _i64, ctypes.POINTER(_int), ctypes.POINTER(_int)]),
     "trsm_wait_selftest": (_int, [_int, _i64, _vp]),
     "trsm_residual_sliced": (_int, [_dp, _i64, _i64, _dp, _i64, _i64, _dp, _i64, _dp, _i64, _int, _vp, _vp]),
     "trsm_residual_plan": (_int, [_vp, _dp, _i64, _i64, _dp, _i64, _dp, _i64, _int, _vp, _vp]),

@@ -10,6 +10,7 @@
 
 #include "internal.h"
 #include "trsm_gb300.h"
+#include "trsm_gb300_engine.h"
 
 
 namespace {
@@ -236,6 +237,32 @@ int trsm_solve(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, dou
   e = trsm::solve_any(h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, ws, h->status, s);
   cudaError_t e2 = trsm::ws_free(ws, s);
   return from_cuda(e != cudaSuccess ? e : e2);
+}
+
+int trsm_solve_form(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, double* X_dev, int64_t ldx, int S,
+                    int CW, void* stream) {
+  int rc = check_solve_args(h, B_dev, k, ldb, X_dev, ldx);
+  if (rc != TRSM_SUCCESS || k == 0) return rc;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (S != 0 || CW != 0) {
+    const trsm::ColPlan p = trsm::col_plan_as(h->n, h->n0, k, S, CW);
+    if (p.S == 0) return TRSM_EINVAL;
+    return from_cuda(trsm::col_solve(p, h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, h->status, s));
+  }
+  void* ws = nullptr;
+  cudaError_t e = trsm::ws_alloc(&ws, trsm::solve_workspace_bytes(h->n, h->n0, k), s);
+  if (e != cudaSuccess) return from_cuda(e);
+  e = trsm::solve_enqueue(h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, ws, h->status, s);
+  cudaError_t e2 = trsm::ws_free(ws, s);
+  return from_cuda(e != cudaSuccess ? e : e2);
+}
+
+int trsm_solve_form_choice(trsm_handle_t h, int64_t k, int* S, int* CW) {
+  if (!h || k < 1 || !S || !CW) return TRSM_EINVAL;
+  const trsm::ColPlan p = trsm::col_plan(h->n, h->n0, k);
+  *S = p.use ? p.S : 0;
+  *CW = p.use ? p.CW : 0;
+  return TRSM_SUCCESS;
 }
 
 int trsm_host(const double* L_host, int64_t n, int64_t ldl, int64_t n0, const double* B_host,

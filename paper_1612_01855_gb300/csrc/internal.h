@@ -84,6 +84,8 @@ struct ColPlan {
   size_t smem = 0;
 };
 ColPlan col_plan(int64_t n, int64_t n0, int64_t k);
+// The plan with a given S and CW; S is 0 where that cannot run.
+ColPlan col_plan_as(int64_t n, int64_t n0, int64_t k, int S, int CW);
 cudaError_t col_solve(const ColPlan& p, const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B, int64_t k,
                       int64_t ldb, double* X, int64_t ldx, int* status_dev, cudaStream_t s);
 

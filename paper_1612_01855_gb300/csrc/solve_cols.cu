@@ -369,22 +369,54 @@ int resident_clusters(int S) {
 
 }  // namespace
 
+namespace {
+
+// The block orders that run by columns: a row group per warp, whole 16-byte
+// pairs of rows in every column.
+bool cols_ok(int64_t n0, int64_t N) { return n0 <= kMaxRows && (N == 1 || n0 % 2 == 0) && N <= 1 << 20; }
+
+// One way to run: S CTAs on CW columns.  S is 0 where their rows do not fit.
+struct ColShape {
+  ColPlan plan;
+  double share = 0;       // column groups an SM (of S, a cluster) takes
+  bool together = false;  // CTAs of more than one on an SM at a time
+};
+ColShape col_shape(int64_t n0, int64_t N, int64_t k, int S, int CW) {
+  ColShape c;
+  const size_t fixed = fixed_bytes(n0, N, S, CW);
+  constexpr size_t kStage = kStageDoubles * sizeof(double);
+  if (fixed + 2 * kStage > kMaxShared) return c;
+  c.share = std::ceil(static_cast<double>((k + CW - 1) / CW) / resident_clusters(S));
+  const size_t room = c.share > 1 ? kMaxShared / 2 : kMaxShared;  // two CTAs on an SM where there are more
+  // (their registers too: 102 a thread for 18 warps)
+  c.together = fixed + 2 * kStage <= room && (c.share <= 1 || CW <= 6);
+  c.plan.S = S;
+  c.plan.CW = CW;
+  c.plan.stages = static_cast<int>(std::min<size_t>(((c.together ? room : kMaxShared) - fixed) / kStage, kMaxStages));
+  c.plan.smem = fixed + c.plan.stages * kStage;
+  return c;
+}
+
+}  // namespace
+
+ColPlan col_plan_as(int64_t n, int64_t n0, int64_t k, int S, int CW) {
+  const int64_t N = (n + n0 - 1) / n0;
+  if (!cols_ok(n0, N) || S < 1 || S > kMaxCluster || S > N || CW < 1 || CW > kMaxCols) return ColPlan();
+  return col_shape(n0, N, k, S, CW).plan;
+}
+
 ColPlan col_plan(int64_t n, int64_t n0, int64_t k) {
   ColPlan best;
   const int64_t N = (n + n0 - 1) / n0;
-  // a row group per warp; whole 16-byte pairs of rows in every column
-  if (n0 > kMaxRows || (N > 1 && n0 % 2 != 0) || N > 1 << 20) return best;
+  if (!cols_ok(n0, N)) return best;
   const int RG = static_cast<int>((n0 + 31) / 32);
   double t_best = 1e300;
   for (int S = 1; S <= kMaxCluster && S <= N; ++S) {
     for (int CW = 1; CW <= kMaxCols; ++CW) {
-      const size_t fixed = fixed_bytes(n0, N, S, CW);
-      constexpr size_t kStage = kStageDoubles * sizeof(double);
-      if (fixed + 2 * kStage > kMaxShared) continue;
-      const double share = std::ceil(static_cast<double>((k + CW - 1) / CW) / resident_clusters(S));
-      const size_t room = share > 1 ? kMaxShared / 2 : kMaxShared;  // two CTAs on an SM where there are more
-      // (their registers too: 102 a thread for 18 warps)
-      const bool together = fixed + 2 * kStage <= room && (share <= 1 || CW <= 6);
+      const ColShape shape = col_shape(n0, N, k, S, CW);
+      if (shape.plan.S == 0) continue;
+      const double share = shape.share;
+      const bool together = shape.together;
       // Clocks.  Throughput: the multiply-adds at 2 per clock (1.12 times
       // that for one or two columns: the loads of L~) and the reductions of
       // the own block rows.  The chain of block rows: two products of order
@@ -401,10 +433,7 @@ ColPlan col_plan(int64_t n, int64_t n0, int64_t k) {
       const double t = std::max(work, rounds * chain) + 0.25 * std::min(work, rounds * chain);
       if (t < t_best) {
         t_best = t;
-        best.S = S;
-        best.CW = CW;
-        best.stages = static_cast<int>(std::min<size_t>(((together ? room : kMaxShared) - fixed) / kStage, kMaxStages));
-        best.smem = fixed + best.stages * kStage;
+        best = shape.plan;
       }
     }
   }
