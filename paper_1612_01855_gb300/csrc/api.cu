@@ -216,8 +216,8 @@ int trsm_solve_ws(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, 
   if (rc != TRSM_SUCCESS || k == 0) return rc;
   const size_t need = trsm::solve_workspace_bytes(h->n, h->n0, k);
   if (!ws_dev || ws_bytes < need || ((uintptr_t)ws_dev % 256) != 0) return TRSM_EINVAL;
-  return from_cuda(trsm::solve_any(h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx,
-                                       ws_dev, h->status, (cudaStream_t)stream));
+  return from_cuda(trsm::solve_any(trsm::col_plan(h->n, h->n0, k), h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx,
+                                   ws_dev, h->status, (cudaStream_t)stream));
 }
 
 int trsm_solve(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, double* X_dev,
@@ -226,15 +226,18 @@ int trsm_solve(trsm_handle_t h, const double* B_dev, int64_t k, int64_t ldb, dou
   if (rc != TRSM_SUCCESS || k == 0) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t need = trsm::solve_workspace_bytes(h->n, h->n0, k);
-  // The solve by columns needs no workspace.  Small ones do without the
-  // pool's allocate and free, about 8 of their 20 us; for the others the
-  // pool keeps what a solve of their size reserves under either form.
-  if (need <= (size_t)1 << 20 && trsm::col_plan(h->n, h->n0, k).use)
-    return from_cuda(trsm::solve_any(h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, nullptr, h->status, s));
+  const trsm::ColPlan cols = trsm::col_plan(h->n, h->n0, k);
+  // The solve by columns uses no workspace.  Small ones do without the pool's
+  // allocate and free, about 8 of their 20 us.  Above 1 MiB, where that is no
+  // longer seen, it is taken all the same: what a solve of n and k leaves
+  // reserved, and so the memory a program finds when it repeats it, does not
+  // depend on the rule.
+  if (need <= (size_t)1 << 20 && cols.use)
+    return from_cuda(trsm::solve_any(cols, h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, nullptr, h->status, s));
   void* ws = nullptr;
   cudaError_t e = trsm::ws_alloc(&ws, need, s);
   if (e != cudaSuccess) return from_cuda(e);
-  e = trsm::solve_any(h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, ws, h->status, s);
+  e = trsm::solve_any(cols, h->Lt, h->ldt, h->n, h->n0, B_dev, k, ldb, X_dev, ldx, ws, h->status, s);
   cudaError_t e2 = trsm::ws_free(ws, s);
   return from_cuda(e != cudaSuccess ? e : e2);
 }

@@ -89,10 +89,10 @@ ColPlan col_plan_as(int64_t n, int64_t n0, int64_t k, int S, int CW);
 cudaError_t col_solve(const ColPlan& p, const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B, int64_t k,
                       int64_t ldb, double* X, int64_t ldx, int* status_dev, cudaStream_t s);
 
-// The solve by whichever of the two is expected to be faster; ws may be null
-// when col_plan says use.
-cudaError_t solve_any(const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B, int64_t k, int64_t ldb,
-                      double* X, int64_t ldx, void* ws, int* status_dev, cudaStream_t s);
+// The solve by whichever of the two is expected to be faster (cols is col_plan
+// of n, n0 and k); ws may be null when that is the one by columns.
+cudaError_t solve_any(const ColPlan& cols, const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B,
+                      int64_t k, int64_t ldb, double* X, int64_t ldx, void* ws, int* status_dev, cudaStream_t s);
 
 // Device status word and device ordinal of a plan (for entry points that
 // live outside api.cu).

@@ -88,7 +88,7 @@ extern "C" int trsm_solve_noalloc(trsm_handle_t h, const double* B_dev, int64_t 
   }
   int64_t ldt = 0;
   const double* Lt = trsm_plan_lt(h, &ldt);
-  e = trsm::solve_any(Lt, ldt, n, n0, B_dev, k, ldb, X_dev, ldx, ws, trsm::plan_status_word(h),
+  e = trsm::solve_any(trsm::col_plan(n, n0, k), Lt, ldt, n, n0, B_dev, k, ldb, X_dev, ldx, ws, trsm::plan_status_word(h),
                           (cudaStream_t)stream);
   if (e != cudaSuccess) {
     cudaGetLastError();

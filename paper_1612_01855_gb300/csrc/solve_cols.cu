@@ -412,22 +412,29 @@ ColPlan col_plan(int64_t n, int64_t n0, int64_t k) {
   const int RG = static_cast<int>((n0 + 31) / 32);
   double t_best = 1e300;
   for (int S = 1; S <= kMaxCluster && S <= N; ++S) {
-    for (int CW = 1; CW <= kMaxCols; ++CW) {
+    for (int CW = 1; CW <= kMaxCols && CW <= k; ++CW) {
       const ColShape shape = col_shape(n0, N, k, S, CW);
       if (shape.plan.S == 0) continue;
       const double share = shape.share;
       const bool together = shape.together;
       // Clocks.  Throughput: the multiply-adds at 2 per clock (1.12 times
       // that for one or two columns: the loads of L~) and the reductions of
-      // the own block rows.  The chain of block rows: two products of order
-      // n0, one dependent multiply-add every 125 clocks or their throughput,
-      // and a signal.  What a CTA alone on its SM waits for its own part of
-      // the chain is lost; of the shorter of the two a quarter shows.
-      const double rows = static_cast<double>(n0) * N, b = 32.0 * RG, own = static_cast<double>(N) / S;
-      const double busy = (CW <= 2 ? 1.12 : 1.0) * CW * (0.25 * rows + 0.25 * b) * rows / S + own * 3000.0;
-      const double product = 0.75 * b * b * CW, step = std::max(250.0 * b, product);
-      const double lost = share > 1 && together ? 0.0 : own * (step - product);
-      const double chain = S > 1 ? N * (step + 3000.0) : 0.0;
+      // the own block rows.  upd: a block of an update; diag: a diagonal
+      // product, whose row groups stop at their own last column.  The chain of
+      // block rows: the two one after the other (the first row has its
+      // diagonal product alone), one dependent multiply-add every 125 clocks or
+      // their throughput, and a signal.  What a CTA alone on its SM waits for
+      // its own part of the chain is lost, beyond the throughput that is
+      // counted already, and its start too; of the shorter of work and chain a
+      // quarter shows.
+      const double b = 32.0 * RG, own = static_cast<double>(N) / S;
+      const double upd = 0.5 * b * b * CW, diag = 0.25 * b * (b + 32) * CW;
+      const double busy = (CW <= 2 ? 1.12 : 1.0) * (0.5 * N * (N - 1) * upd + N * diag) / S + own * 3000.0;
+      const double first = std::max(125.0 * b, diag), step = std::max(250.0 * b, upd + diag);
+      const double lost = share > 1 && together
+                              ? 0.0
+                              : ((N - 1) * (step - upd - diag) + first - diag) / S + (share > 1 ? 2000.0 : 0.0);
+      const double chain = S > 1 ? (N - 1) * (step + 3000.0) + first + 3000.0 : 0.0;
       const double rounds = together ? std::ceil(share / 2) : share;
       const double work = share * (busy + (S > 1 ? 0.0 : lost));
       const double t = std::max(work, rounds * chain) + 0.25 * std::min(work, rounds * chain);
@@ -445,7 +452,11 @@ ColPlan col_plan(int64_t n, int64_t n0, int64_t k) {
   // 1258, 512 x 512 538 / 206, 1000 x 200 1026 / 294, 1000 x 37 1001 / 159;
   // n0 = 256, 2048 x 500 2914 / 2280, 4096 x 150 4849 / 2540, 4096 x 400 7284 /
   // 6655, 4096 x 800 11890 / 13220, 8192 x 64 9071 / 5262, 8192 x 152 12570 /
-  // 9896, 8192 x 300 19400 / 17420.
+  // 9896, 8192 x 300 19400 / 17420, 3017 x 507 5163 / 4709, 1454 x 1147 2720 /
+  // 2509, 1112 x 988 1741 / 1530.  Below n = 300 the division matters more than
+  // the form (us by columns a group, one CTA each): 64 x 1 8.4 / 8.4 / 8.4 / - /
+  // 12.4 for 1, 2, 3, 5 of them, 64 x 4 the same, 64 x 8 the same, 128 x 1 at
+  // n0 = 128 11.2 for 1, 17.4 for 3, 7 x 1 4.5 for 1, 5.1 for 8.
   const double tiles =
       0.25 * static_cast<double>(n) * n * static_cast<double>((k + 31) / 32 * 32) / device_sm_count();
   const double tile_chain = N * (2.0 * RG * 16400 + 30000);
@@ -488,9 +499,8 @@ cudaError_t col_solve(const ColPlan& p, const double* Lt, int64_t ldt, int64_t n
   }
 }
 
-cudaError_t solve_any(const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B, int64_t k, int64_t ldb,
-                      double* X, int64_t ldx, void* ws, int* status_dev, cudaStream_t s) {
-  const ColPlan cols = col_plan(n, n0, k);
+cudaError_t solve_any(const ColPlan& cols, const double* Lt, int64_t ldt, int64_t n, int64_t n0, const double* B,
+                      int64_t k, int64_t ldb, double* X, int64_t ldx, void* ws, int* status_dev, cudaStream_t s) {
   if (cols.use) return col_solve(cols, Lt, ldt, n, n0, B, k, ldb, X, ldx, status_dev, s);
   return solve_enqueue(Lt, ldt, n, n0, B, k, ldb, X, ldx, ws, status_dev, s);
 }

@@ -78,3 +78,15 @@ def test_choice_and_arguments(cuda_lib):
         assert _solve(cuda_lib, plan, Bd, Bd.clone(), S, CW) == -1
     assert cuda_lib.trsm_solve_form(None, None, 1, 1, None, 1, 0, 0, None) == -1
     assert cuda_lib.trsm_solve_form_choice(None, 1, None, None) == -1
+
+
+@pytest.mark.parametrize("n,n0", [(2, 2), (64, 64), (128, 64), (128, 128), (1000, 64), (1272, 256)])
+def test_no_more_columns_a_group_than_there_are(cuda_lib, n, n0):
+    """A group wider than the right-hand side would solve columns of zeros."""
+    import paper_1612_01855_gb300 as g
+    L, _ = inputs.well_conditioned(n, 1, seed=2)
+    plan = g.trsm_plan(_dev(L), n0)
+    S, CW = ctypes.c_int(-1), ctypes.c_int(-1)
+    for k in range(1, 9):
+        assert cuda_lib.trsm_solve_form_choice(plan.handle, k, ctypes.byref(S), ctypes.byref(CW)) == 0
+        assert S.value >= 1 and 1 <= CW.value <= k, (k, S.value, CW.value)
