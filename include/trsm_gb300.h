@@ -371,16 +371,16 @@ size_t trsm_plan_device_bytes(trsm_handle_t h);
  * call frees stays reserved in the pool for the next call (the device's
  * default pool would unmap it at each synchronisation and the next call
  * would map it again, about 1 ms per GB), and is not handed to another
- * stream before its free has completed there.  A second pool holds the L~
- * of plans of up to 32 MiB, which destroying the plan leaves reserved for
- * the next one.  No counterpart in the paper.
+ * stream before its free has completed there.  L~ of a plan of up to 32 MiB
+ * lies in a block that destroying the plan leaves to the next one of its
+ * size (at most 256 MiB idle in all).  No counterpart in the paper.
  *   trsm_workspace_trim: returns the current device's idle pool memory to
  *     the system until at most keep_bytes stay reserved (memory of calls
  *     still in flight and of plans stays).  TRSM_SUCCESS, also when never
  *     used; TRSM_ECUDA without a usable device.  An allocation the pool
  *     cannot satisfy trims the pool itself and retries once.
- *   trsm_workspace_reserved_bytes: bytes the current device's pools hold
- *     mapped (in use or idle); 0 without a device or before the first call. */
+ *   trsm_workspace_reserved_bytes: bytes the current device's pool and those
+ *     blocks hold mapped (in use or idle); 0 without a device or before the first call. */
 int trsm_workspace_trim(size_t keep_bytes);
 size_t trsm_workspace_reserved_bytes(void);
 

@@ -40,23 +40,23 @@ std::vector<trsm::DiagBlock> diag_blocks(int64_t n, int64_t n0, int64_t ld, bool
   return v;
 }
 
-// Memory of L~.  Small plans take it from a pool instead of mapping and
-// unmapping fresh memory (cudaMalloc, cudaFree): at n = 512 a plan and its
-// destruction took 250 and 105 us, 90 and 4 us so, with no wait for the
-// descriptors' copy.  The line lies where that mapping stops mattering beside
-// the solves a plan is made for (134 MB, n = 4096: 112 of 1200 us for a plan
-// and a solve of 16 columns go into its destruction) and bounds what idles in
-// the pool (pool.cu).  A capturing stream, on which a plan cannot be made,
+// Memory of L~.  Small plans take a block that a destroyed plan left instead
+// of mapping and unmapping fresh memory (cudaMalloc, cudaFree): at n = 512 a
+// plan and its destruction took 250 and 105 us, 90 and 4 us so, with no wait
+// for the descriptors' copy.  The line lies where that mapping stops mattering
+// beside the solves a plan is made for (134 MB, n = 4096: 112 of 1200 us for a
+// plan and a solve of 16 columns go into its destruction); what idles is
+// bounded in pool.cu.  A capturing stream, on which a plan cannot be made,
 // fails as it does with cudaMalloc.
-constexpr size_t kPoolPlanBytes = (size_t)32 << 20;
-cudaError_t alloc_lt(double** p, size_t bytes, cudaStream_t s) {
+constexpr size_t kBlockPlanBytes = (size_t)32 << 20;
+cudaError_t alloc_lt(trsm_plan_s* h, size_t bytes, cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-  if (bytes <= kPoolPlanBytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+  if (bytes <= kBlockPlanBytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
     trsm::keep_small_block();
-    return trsm::plan_alloc((void**)p, bytes, s);
+    return trsm::plan_alloc((void**)&h->Lt, bytes, &h->lt_block);
   }
   cudaGetLastError();
-  return cudaMalloc((void**)p, bytes);
+  return cudaMalloc((void**)&h->Lt, bytes);
 }
 
 // Inverts the listed blocks and reports a singular pivot.  Synchronous.
@@ -182,7 +182,7 @@ int trsm_plan(const double* L_dev, int64_t n, int64_t ldl, int64_t n0, void* str
   h->ldt = align4(n);
   cudaGetDevice(&h->device);
   cudaError_t e = cudaMalloc((void**)&h->status, sizeof(int));
-  if (e == cudaSuccess) e = alloc_lt(&h->Lt, sizeof(double) * (size_t)h->ldt * (size_t)n, s);
+  if (e == cudaSuccess) e = alloc_lt(h, sizeof(double) * (size_t)h->ldt * (size_t)n, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), s);
   if (e == cudaSuccess) e = trsm::copy_lower(L_dev, ldl, h->Lt, h->ldt, n, s);
   int rc = from_cuda(e);
@@ -384,11 +384,15 @@ void trsm_destroy(trsm_handle_t h) {
   int cur = 0;
   cudaGetDevice(&cur);
   if (cur != h->device) cudaSetDevice(h->device);
-  // The cudaFree of the status word, which is cudaMalloc's, waits for the
-  // device work that may still use the plan; that of L~ need not wait (where
-  // it is the pool's) or waits again.
-  if (h->status) cudaFree(h->status);
-  if (h->Lt) cudaFree(h->Lt);
+  // The cudaFree of the status word returns when the device has finished all
+  // work that may use the plan (26 ms beside a kernel of that length, with
+  // nothing to unmap; a test holds it to that), so that L~'s block may go to
+  // the next plan.  A cudaDeviceSynchronize in its place would end another
+  // thread's capture, which a cudaFree leaves alone unless the capture is a
+  // global one; a cudaFree that fails, in such a capture, has not waited.
+  const bool unused = !h->status || cudaFree(h->status) == cudaSuccess;
+  if (h->Lt && h->lt_block.bytes) trsm::plan_free(h->Lt, h->lt_block, unused);
+  else if (h->Lt) cudaFree(h->Lt);
   trsm::mixed_release(h);
   trsm::sliced_release(h);
   if (cur != h->device) cudaSetDevice(cur);

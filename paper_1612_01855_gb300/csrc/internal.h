@@ -10,6 +10,11 @@
 namespace trsm {
 struct MixedPlan;
 struct SlicedPlan;
+// A block of device memory that passes from plan to plan (pool.cu); 0 bytes: none.
+struct PlanBlock {
+  size_t bytes = 0;
+  unsigned long long ctx_id = 0;  // context it was made in
+};
 }
 
 // The plan behind trsm_handle_t.
@@ -18,6 +23,7 @@ struct trsm_plan_s {
   double* Lt = nullptr;   // L~: n x n, leading dimension ldt
   int* status = nullptr;  // sticky device status of solves
   int device = 0;
+  trsm::PlanBlock lt_block;  // where Lt is a block of plan_alloc
   trsm::MixedPlan* mixed = nullptr;    // low-precision data (trsm_plan_mixed), or null
   trsm::SlicedPlan* sliced = nullptr;  // residues of the sliced schedule (trsm_plan_sliced), or null
 };
@@ -106,9 +112,12 @@ int plan_device(trsm_handle_t h);
 // mapping again at each call (about 1 ms per GB).  trsm_workspace_trim
 // returns the pool's idle memory (pool.cu).
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
-// The same from a pool for plans, to be freed by cudaFree once its last use
-// is over; keep_small_block makes cudaMalloc and cudaFree of single words cheap.
-cudaError_t plan_alloc(void** p, size_t bytes, cudaStream_t s);
+// Memory of a plan, cudaMalloc's, from the blocks that destroyed plans left
+// where one fits.  plan_free gives it back; unused: the device has finished all
+// work that may use it, so that the next plan may have it.  keep_small_block
+// makes cudaMalloc and cudaFree of single words cheap.
+cudaError_t plan_alloc(void** p, size_t bytes, PlanBlock* block);
+void plan_free(void* p, const PlanBlock& block, bool unused);
 void keep_small_block();
 cudaError_t ws_free(void* p, cudaStream_t s);
 template <class T>
