@@ -963,7 +963,8 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   const int64_t ld = trsm::align4(n);
   const size_t esz = trsm::mode_bytes(mode);
 
-  // workspace: R, D (FP64), W (FP32), Dt (low precision), residues of X and of the products, norms, error word
+  // workspace: R, D (FP64), W (FP32), Dt (low precision), residues of X and of
+  // the products (none for the FP64 residual), norms, error word
   size_t off = 0;
   const size_t oR = off;
   off = trsm::align256(off + sizeof(double) * ld * k);
@@ -974,9 +975,10 @@ extern "C" int trsm_solve_mixed(trsm_handle_t h, const double* B_dev, int64_t k,
   const size_t oDt = off;
   off = trsm::align256(off + esz * n0p * k);
   const size_t oXs = off;
-  off = trsm::align256(off + trsm::rns_operand_bytes(k, n));
+  const bool rns = residual != TRSM_RESIDUAL_FP64;
+  off = trsm::align256(off + (rns ? trsm::rns_operand_bytes(k, n) : 0));
   const size_t oPart = off;
-  off = trsm::align256(off + (residual != TRSM_RESIDUAL_FP64 ? trsm::rns_scratch_bytes(n, k) : 0));
+  off = trsm::align256(off + (rns ? trsm::rns_scratch_bytes(n, k) : 0));
   const size_t oErr = off;
   off = trsm::align256(off + sizeof(int));
   const size_t oDmax = off;  // per block row: max |D_i| (split fp16 scaling); then max |D|, max |X|
