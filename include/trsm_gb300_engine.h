@@ -76,7 +76,11 @@ int trsm_solve_form_choice(trsm_handle_t h, int64_t k, int* S, int* CW);
  *             batched solve kernels, on a counter nothing raises;
  *   kind = 1: an mbarrier wait, the routine of the tcgen05 kernels, on a
  *             barrier that never gets its arrival, in a CTA holding tensor
- *             memory (freed before it returns).
+ *             memory (freed before it returns);
+ *   kind = 3: a copy ring whose consumer gives no stage back, the loader of
+ *             the solve by columns and of the tcgen05 kernels, which drains
+ *             the copies it has issued before it returns;
+ *   kind = 4: a wait for another CTA of a cluster, as in the solve by columns.
  * Returns TRSM_ETIMEOUT when the wait ran out and the kernel drained (the
  * expected outcome: the device stays usable), TRSM_SUCCESS if it did not,
  * TRSM_EINVAL or TRSM_ECUDA.  Synchronous on `stream`. */

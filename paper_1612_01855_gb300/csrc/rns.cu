@@ -739,6 +739,10 @@ __global__ void __maxnreg__(kMaxRegs)
           }
         }
       }
+      // A pair's copies complete on the leader's barriers alone, so the leader
+      // waits for both CTAs'; the other one's are no later than its wait that
+      // gave up, hundreds of polls.
+      if (!ok && rank == 0) tc::drain_ring(full_bar, STAGES, it);
       // the leader's last commits have landed here before this CTA may end
       if constexpr (kPair)
         for (int i = max(0, it - STAGES); ok && i < it; ++i)

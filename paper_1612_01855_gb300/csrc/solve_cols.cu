@@ -62,36 +62,9 @@ struct ColArgs {
   int* status;
 };
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(tc::smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(tc::smem_u32(bar))
-      : "memory");
-}
-
 // Barrier among the consumers.
 __device__ __forceinline__ void sync_consumers() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarps) : "memory");
-}
-
-// Waits for an arrival of the other CTAs of the cluster (acquire at cluster
-// scope); false when the wait gave up (bounded as every wait) or the CTA is
-// aborting.
-__device__ __forceinline__ bool wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  const long long t0 = tc::globaltimer_ns();
-  for (uint32_t i = 0; i < tc::kMbarSpinLimit; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(tc::smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if ((i & 255u) == 255u && (*abort_flag || tc::globaltimer_ns() - t0 > tc::kMbarWaitNs)) break;
-  }
-  return false;
 }
 
 __device__ __forceinline__ void st_cluster(uint32_t addr, double v) {
@@ -172,8 +145,8 @@ __global__ void __launch_bounds__(kThreads, 1) col_solve_kernel(const ColArgs a)
         const uint32_t b = static_cast<uint32_t>((rows_of(l) + 1) / 2 * 16);
         double* dst = sm + static_cast<size_t>(q) * kStageDoubles + static_cast<size_t>((t - base) * kc) * a.pitch;
         for (int c = lane; c < cols; c += 32)
-          bulk_load(dst + static_cast<size_t>(c) * a.pitch, a.Lt + (c0 + c) * a.ldt + static_cast<int64_t>(l) * a.n0, b,
-                    &full_bar[q]);
+          tc::bulk_load(dst + static_cast<size_t>(c) * a.pitch, a.Lt + (c0 + c) * a.ldt + static_cast<int64_t>(l) * a.n0, b,
+                        &full_bar[q]);
       }
       ++it;
     };
@@ -194,6 +167,7 @@ __global__ void __launch_bounds__(kThreads, 1) col_solve_kernel(const ColArgs a)
           stage(static_cast<int64_t>(b) * a.n0 + q, min(a.KCn, a.n0 - q), max(t0, g * a.NB), min(own, (g + 1) * a.NB),
                 g * a.NB, a.KCn);
     }
+    if (!ok && lane == 0) tc::drain_ring(full_bar, a.stages, it);
   } else {
     int it = 0;
     bool ok = true;
@@ -265,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1) col_solve_kernel(const ColArgs a)
     for (int b = 0; b + 1 < a.N; ++b) {
       const int slot = b % (S + 1);
       const double* x = xs + static_cast<size_t>(slot) * block_doubles;
-      if (!wait_cluster(&x_bar[slot], (b / (S + 1)) & 1, abort_flag)) *abort_flag = 1;
+      tc::mbar_wait_cluster(&x_bar[slot], (b / (S + 1)) & 1, abort_flag, tc::kMbarWaitNs);
       if ((b + 1) % S == rank) {
         const int l = b + 1, ml = rows_of(l);
         double* w = W + static_cast<size_t>(l / S) * block_doubles;

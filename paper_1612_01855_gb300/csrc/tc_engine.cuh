@@ -20,6 +20,7 @@ namespace tc {
 // hardware time slice per poll) or kMbarSpinLimit polls, whichever is first.
 constexpr uint32_t kMbarSpinLimit = 1u << 26;
 constexpr long long kMbarWaitNs = 2000000000LL;
+constexpr long long kDrainNs = 100000000LL;  // for copies under way when a role gives up
 
 __device__ __forceinline__ long long globaltimer_ns() {
   long long t;
@@ -80,6 +81,44 @@ __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, 
 
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   return mbar_wait_limit(bar, parity, abort_flag, kMbarWaitNs);
+}
+
+// Untiled copy of `bytes` (a multiple of 16, as both addresses) into this CTA.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// For a role that gives up after it has issued `issued` stages of a ring of
+// `stages` full barriers: waits for the copies still under way, with a limit
+// of its own, so that the CTA does not end with copies into its shared memory.
+__device__ __forceinline__ void drain_ring(uint64_t* full_bar, int stages, int issued) {
+  int gave_up = 0;
+  for (int i = issued > stages ? issued - stages : 0; i < issued && !gave_up; ++i)
+    mbar_wait_limit(&full_bar[i % stages], (i / stages) & 1, &gave_up, kDrainNs);
+}
+
+// As mbar_wait_limit for arrivals of other CTAs of the cluster (acquire at
+// cluster scope).
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                  long long limit_ns) {
+  const long long t0 = globaltimer_ns();
+  for (uint32_t i = 0; i < kMbarSpinLimit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((i & 255u) == 255u && (*abort_flag || globaltimer_ns() - t0 > limit_ns)) break;
+  }
+  *abort_flag = 1;
+  return false;
 }
 
 // 3-D TMA tile load (coordinates: x = K offset in elements, y = row, z = slice).

@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(192, 1)
         }
         if (!ok) break;
       }
+      if (*abort_flag) drain_ring(full_bar, STAGES, it);
     }
   } else if (warp == 1) {
     if (lane == 0) {
