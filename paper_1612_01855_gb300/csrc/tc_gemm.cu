@@ -65,7 +65,6 @@ struct StoreF32Epi {
   int M, N, nkb;
   float alpha, beta;
   const float* scale = nullptr;  // optional device factor on alpha (set by an earlier kernel)
-  struct State {};
   // Launch order -> tile: groups of kGroupRows row tiles, within a group the
   // column tiles one after the other.  The CTAs in flight (one per SM) then
   // cover about 16 row tiles x 10 column tiles, whose A and B panels stay
@@ -79,17 +78,11 @@ struct StoreF32Epi {
     tm = g0 + idx % gsz;
     tn = idx / gsz;
   }
-  __device__ void tile(int& tm, int& tn) const {
-    const int R = static_cast<int>(gridDim.x), C = static_cast<int>(gridDim.y);
-    tile_of(tm + R * tn, R, C, tm, tn);
-  }
-  __device__ void k_range(int, int, int& kb0, int& kb1, int& chunk) const {
+  __device__ void k_range(int, int, int& kb0, int& kb1) const {
     kb0 = 0;
     kb1 = nkb;
-    chunk = nkb > 0 ? nkb : 1;
   }
-  __device__ void init(State&) const {}
-  __device__ void group(State&, int tm, int tn, int, int row, int sl, int, const float (&v)[16]) const {
+  __device__ void group(int tm, int tn, int row, int sl, int, const float (&v)[16]) const {
     const int r = tm * 128 + row;
     if (r >= M) return;
     float* base = C + static_cast<int64_t>(tn * BN + sl * 16) * ldc + r;
@@ -103,8 +96,6 @@ struct StoreF32Epi {
     for (int j = 0; j < 16; ++j)
       if (j < ncol) base[static_cast<int64_t>(j) * ldc] = a * v[j] + beta * old[j];
   }
-  __device__ void slab_done(State&, int, int, int, int, int) const {}
-  __device__ void finish(State&, int, int, int, int) const {}
 };
 
 // D (FP64, column-major, ldd) = A B^T with a single FP32 group (the
@@ -120,7 +111,6 @@ struct StoreF64MaxEpi {
   int M, N, K;
   int lower;
   unsigned long long* dmax;
-  struct State {};
   // Launch order -> tile: the row tiles from the last (longest sums) to the
   // first, each over all its column tiles.  In the persistent kernel CTA c
   // takes the tiles t = c, c + G, c + 2G, ... (G CTAs); lower triangular
@@ -141,21 +131,12 @@ struct StoreF64MaxEpi {
       tn = lin / R;
     }
   }
-  __device__ void tile(int& tm, int& tn) const {
-    if (!lower) return;
-    const int R = static_cast<int>(gridDim.x), C = static_cast<int>(gridDim.y);
-    const int lin = tm + R * tn;
-    tm = R - 1 - lin / C;
-    tn = lin % C;
-  }
-  __device__ void k_range(int tm, int, int& kb0, int& kb1, int& chunk) const {
+  __device__ void k_range(int tm, int, int& kb0, int& kb1) const {
     const int kend = lower ? min(K, (tm + 1) * 128) : K;
     kb0 = 0;
     kb1 = (kend + KB - 1) / KB;
-    chunk = kb1 > 0 ? kb1 : 1;
   }
-  __device__ void init(State&) const {}
-  __device__ void group(State&, int tm, int tn, int, int row, int sl, int, const float (&v)[16]) const {
+  __device__ void group(int tm, int tn, int row, int sl, int, const float (&v)[16]) const {
     const int r = tm * 128 + row;
     const int c0 = tn * BN + sl * 16;
     const int ncol = (r < M) ? min(16, N - c0) : 0;
@@ -180,8 +161,6 @@ struct StoreF64MaxEpi {
                                                          static_cast<double>(__uint_as_float(mf))));
     if ((threadIdx.x & 31) == 0 && mb) atomicMax(dmax, mb);
   }
-  __device__ void slab_done(State&, int, int, int, int, int) const {}
-  __device__ void finish(State&, int, int, int, int) const {}
 };
 
 // Launches the persistent tile kernel over the R x C tiles: as many CTAs as
