@@ -168,7 +168,8 @@ int trsm_solve_schedule(trsm_handle_t h, const double* B_dev, int64_t k, int64_t
  * applied to the two matrix multiplies of It-Inv-TRSM, Section 6.2).  From
  * the plan's L~ it makes the bf16 residues modulo 15 moduli of L off the
  * diagonal blocks (15 n (n + n0) bytes) and of the rows of the inverted
- * diagonal blocks (30 n n0 bytes), counted by trsm_plan_device_bytes and freed by trsm_destroy.  The block order must
+ * diagonal blocks (30 n n0 bytes), counted by trsm_plan_device_bytes and
+ * freed by trsm_destroy.  The block order must
  * be a multiple of 64 and at most 2048, or the plan a single block (n0 >= n)
  * of order at most 2048 (else TRSM_EINVAL).  A second call is a no-op.
  * Synchronous.  Errors: TRSM_EINVAL, TRSM_ENOMEM, TRSM_ECUDA. */

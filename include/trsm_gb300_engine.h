@@ -36,8 +36,8 @@ int trsm_tc_gemm_selftest(int mode, const void* A_dev, const void* B_dev, float*
  * power-of-two exponent each; their residues modulo 13, 14, 14 or 15 moduli
  * are multiplied with exact FP32 sums, and the chunk's integer product is put
  * together from them (to 3.2 2^-64 of the moduli's product, exactly for
- * factors of up to nine 6-bit digits a pair) and applied in FP64 (after Ozaki, Uchino &
- * Imamura 2025); the diagonal of L is applied in FP64.  Relative error about
+ * factors of up to nine 6-bit digits a pair) and applied in FP64 (after
+ * Ozaki, Uchino & Imamura 2025); the diagonal of L is applied in FP64.  Relative error about
  * 2^-45 (6 or 7 planes) or 2^-50 (8 planes) of (|B| + |L| |X|), about 2^-38
  * with 5.
  *   L_dev n x n column-major (lower triangle read), X_dev, B_dev, R_dev

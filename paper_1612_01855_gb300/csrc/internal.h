@@ -37,8 +37,9 @@ void mixed_release(trsm_plan_s* h);
 // The same for the residues of the sliced schedule.
 size_t sliced_bytes(const trsm_plan_s* h);
 void sliced_release(trsm_plan_s* h);
-// X = L^-1 B by the sliced schedule (sched_sliced.cu): B is copied first, so
-// X may alias B (same leading dimension).
+// X = L^-1 B by the sliced schedule (sched_sliced.cu).  X may alias B (same
+// leading dimension): the first step reads every row of B and keeps the later
+// rows' updates in the workspace before any other row of X is written.
 int solve_sliced(trsm_plan_s* h, const double* B, int64_t k, int64_t ldb, double* X, int64_t ldx,
                  cudaStream_t s);
 

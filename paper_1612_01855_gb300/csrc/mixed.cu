@@ -26,9 +26,9 @@
 //
 // The residual is either the residue-number-system tensor-core product of
 // rns.cu (relative to |B| + |L||X|: about 2^-45 in the seven-plane class,
-// about 2^-50 in the eight-plane class; or seven until the updates stagnate above tol or their
-// contraction stalls, then eight) or
-// a plain FP64 DFMA product.
+// about 2^-50 in the eight-plane class; or seven until the updates stagnate
+// above tol or their contraction stalls, then eight) or a plain FP64 DFMA
+// product.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

@@ -1,8 +1,9 @@
 // Residue-number-system products on the BF16 tensor cores (tcgen05): see
-// rns.h for the method.  Three parts: the residues of an operand
-// (residue_rows_kernel), and the product kernel, whose epilogue reduces each
-// modulus' FP32 sums to bytes and whose last tile per output position puts
-// the integer product together (Chinese remainder theorem) and applies it.
+// rns.h for the method.  Two parts: the residues of an operand
+// (residue_rows_kernel), and the product kernel (rns_product_kernel), whose
+// epilogue reduces each modulus' FP32 sums to bytes and which puts an output
+// tile's integer products together (Chinese remainder theorem) and applies
+// them when its last modulus is there.
 #include <cuda_runtime.h>
 
 #include <algorithm>

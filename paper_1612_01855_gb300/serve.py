@@ -23,8 +23,8 @@ pays for the blocked solve (Algorithm It-Inv-TRSM, Section 6.2).  The loop:
 * with `sliced_min_flops` set, an FP64 request of at least that many n^2 k
   flops whose plan carries the sliced schedule's residues
   (`trsm_plan_sliced`) waits in a third queue and is solved alone on a slot
-  by the sliced schedule (FP64-class products on the tensor cores, 10-20x
-  the DFMA rate on large systems): the largest requests, which set the
+  by the sliced schedule (FP64-class products on the tensor cores, 45-70x
+  the DFMA rate on the largest systems): the largest requests, which set the
   latency tail at the DFMA rate, then take a fraction of the time;
 * between the queues a free slot goes to whichever head arrived first,
   unless that head cannot start (a mixed request while every mixed slot is
